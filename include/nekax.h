@@ -117,9 +117,10 @@ nek_status nek_geom_ff(int64_t nelt, int nx, const double* G, float* Gff, void* 
  * w = AX(u) to FP64 accuracy computed on the FP32 pipes (the operator of
  * Section II-B, Listing 1, in float-float arithmetic).  Same arguments and
  * layouts as nek_ax except Gff (from nek_geom_ff); u, w 8-byte aligned, no
- * overlap.  Every value is carried as a pair of floats (~48 significant bits)
- * and every sum is formed with exact residual tracking; the result matches the
- * FP64 operator to ~1e-14 relative in the max norm.  Element blocks whose
+ * overlap.  Values are carried as pairs of floats (~48 significant bits) or, from
+ * nx = 5 on, as integer digits of the element's largest value with float
+ * remainders whose products are summed exactly; the result matches the
+ * FP64 operator to ~1e-13 relative in the max norm.  Element blocks whose
  * largest |u| is below ~1e-30 (or contain non-finite values) are not covered by
  * that accuracy statement.  Async on stream.
  */
@@ -128,8 +129,9 @@ nek_status nek_ax_ff(int64_t nelt, int nx, const double* D, const float* Gff, co
 
 /*
  * nek_ax_ff plus the element energies edot[e] = u_e . w_e = u_e^T A_e u_e
- * (FP64 products and sums; each element's sum runs in an order fixed by nx
- * alone, so it does not depend on the tuned elements per CTA).  Summed over
+ * (FP64 products; the sums are FP64 in an order fixed by nx alone, from nx = 5 on
+ * with the threads' partial sums added exactly as integers of 2^-53 of the
+ * largest one, so the result does not depend on the tuned elements per CTA).  Summed over
  * elements this is the CG's <p, A p> (Section II-B's inner product of the
  * direction with the assembled operator applied to it) for a p that is
  * continuous across elements and zero on masked nodes; the FP64 solve with

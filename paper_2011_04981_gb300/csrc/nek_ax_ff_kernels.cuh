@@ -1,8 +1,9 @@
-// AX operator to FP64 accuracy on the FP32 pipes (float-float arithmetic).
+// AX operator to FP64 accuracy on the FP32 pipes (float-float arithmetic): the kernel of nx = 2, 3 and 4, the load modes
+// shared with the line-pass kernel of nx >= 5 (nek_ax_fx.cuh), and the launch templates of both.
 //
 // Same operator as nek_ax (Section II-B, Listing 1 of arXiv 2011.04981).  On
 // GB300 the FP64 pipe runs 2 DFMA/clk/SM against 128 FFMA/clk/SM, so native
-// FP64 AX is bound by the FP64 pipe at ~8% of the HBM roofline.  This kernel
+// FP64 AX is bound by the FP64 pipe at ~8% of the HBM roofline.  k_ax_ff
 // keeps every value as an unevaluated pair hi + lo of floats (about 48
 // significant bits) and does all arithmetic on the FP32 pipes, two k-planes per
 // instruction with the packed f32x2 operations of sm_100+.
@@ -23,14 +24,8 @@
 // The pointwise geometric product uses Dekker products (FMA-exact) and Knuth
 // two-sums.  Inputs: u and w in FP64, D in FP64 (split on load), G pre-split by
 // nek_geom_ff into [e][p][12] floats (48 B per point, the same HBM traffic as
-// FP64 G).
-//
-// Two kernel families: k_ax_ff walks (i, j) columns (or groups of planes
-// above nx = 12) with u, wr, ws, wt as float pairs in shared memory; k_ax_ffi
-// (nx = 10 and 12) keeps k-plane pairs as float4 so one load feeds a packed
-// instruction, and spreads an element's (column, k-pair) items over whole
-// warps.  Both take a compile-time load mode (plain, gathered, skipping
-// finished problems, with element energies, with the solve's direction update).
+// FP64 G).  k_ax_ff walks (i, j) columns with u, wr, ws, wt as float pairs in
+// shared memory.
 //
 // This header holds the kernels and their launch templates; the per-nx
 // launchers are compiled in nek_ax_ff_nx_*.cu (a few nx each, so the build's
@@ -180,9 +175,6 @@ struct Lanes<float2> {
     }
 };
 
-template <int NX>
-constexpr int ff_epb();
-
 template <int NX, int EPB>
 constexpr size_t ff_smem_bytes()
 {
@@ -191,36 +183,7 @@ constexpr size_t ff_smem_bytes()
     return sizeof(float2) * (4 * EPB * NX * NX * NX + 2 * NX * NX) + sizeof(float) * (2 * NX + 4 * EPB + 4) + 16;
 }
 
-// k-planes per thread.  Up to nx = 12 a thread walks its whole (i, j) column
-// (measured fastest: the per-thread set-up is amortised over nx planes); above,
-// columns are split into groups of 4 planes (3 at nx = 13) so that one element
-// spreads over up to 1024 threads.
-constexpr int ff_ppt(int nx) { return nx <= 12 ? nx : nx == 13 ? 3 : 4; }
-constexpr int ff_groups(int nx) { return (nx + ff_ppt(nx) - 1) / ff_ppt(nx); }
-constexpr int ff_threads_per_elem(int nx) { return nx * nx * ff_groups(nx); }
-
-// Default elements per CTA: at least ~128 threads per CTA, 1, 2 or 4 where
-// possible; nx = 10 and 12 run the item-mapped kernel with 128 and 144 threads
-// per element, whose measured best counts are 1 and 4 (the tuner may change them).
-template <int NX>
-constexpr int ff_epb()
-{
-    if constexpr (NX == 10) return 1;
-    if constexpr (NX == 12) return 4;
-    return ff_threads_per_elem(NX) >= 128 ? 1 : ff_threads_per_elem(NX) >= 64 ? 2 : 4;
-}
-
-// CTAs per SM the register budget is set for: about 16 resident warps.
-template <int NX, int EPB>
-constexpr int ff_min_blocks()
-{
-    constexpr int warps = (NX * NX * EPB * ff_groups(NX) + 31) / 32;
-    return warps >= 16 ? 1 : (16 / warps > 4 ? 4 : 16 / warps);
-}
-
-// Thread (e, i, j, g) computes the W-wide k-groups of planes [g*PPT, g*PPT + PPT)
-// of element e.
-// Load modes of the float-float kernels: plain w = AX u; GATHER: u is a
+// Load modes of the FP64-accurate kernels: plain w = AX u; GATHER: u is a
 // unique-node vector read through l2g (element point p reads u[l2g[p]]); SKIP:
 // a CTA whose elements all belong to finished problems (eprob: problem of each
 // element, pdone: one byte per problem) returns at once (batched solves); DOT:
@@ -313,7 +276,7 @@ __device__ __forceinline__ double reread_input(int64_t first, int p, const doubl
 }
 
 template <int NX, int EPB, int MODE>
-__global__ void __launch_bounds__(NX* NX* ff_groups(NX)* EPB, (ff_min_blocks<NX, EPB>()))
+__global__ void __launch_bounds__(NX* NX* EPB, 4)
     k_ax_ff(int64_t nelt, const double* __restrict__ D, const float4* __restrict__ Gff,
             const double* __restrict__ u, double* __restrict__ w, const int32_t* __restrict__ l2g,
             const int32_t* __restrict__ eprob, const uint8_t* __restrict__ pdone, double* __restrict__ edot,
@@ -322,9 +285,7 @@ __global__ void __launch_bounds__(NX* NX* ff_groups(NX)* EPB, (ff_min_blocks<NX,
     using T = typename std::conditional<(NX % 2 == 0), float2, float>::type;
     using L = Lanes<T>;
     constexpr int W = L::W;
-    constexpr int PPT = ff_ppt(NX), NG = ff_groups(NX);
-    constexpr int N2 = NX * NX, N3 = NX * NX * NX, TPE = N2 * NG, NT = TPE * EPB;
-    static_assert(PPT % W == 0, "plane groups hold whole k-pairs");
+    constexpr int N2 = NX * NX, N3 = NX * NX * NX, TPE = N2, NT = TPE * EPB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* sU = reinterpret_cast<float2*>(smem_raw);  // [EPB][N3] u (hi, lo)
     float2* sWr = sU + EPB * N3;                       // [EPB][N3] wr
@@ -361,18 +322,14 @@ __global__ void __launch_bounds__(NX* NX* ff_groups(NX)* EPB, (ff_min_blocks<NX,
     }
 
     const int el = tid / TPE;
-    const int q3 = tid - el * TPE;
-    const int g = q3 / N2;
-    const int q2 = q3 - g * N2;
+    const int q2 = tid - el * TPE;
     const int i = q2 % NX, j = q2 / NX;
-    const int kbeg = g * PPT;
-    const int kend = kbeg + PPT < NX ? kbeg + PPT : NX;
     const bool active = el < ne;
     const float2* ue = sU + el * N3;
     {
         float m = 0.f;
         if (active)
-            for (int k = kbeg; k < kend; k++) m = absmax_bits(ue[i + NX * (j + NX * k)].x, m);
+            for (int k = 0; k < NX; k++) m = absmax_bits(ue[i + NX * (j + NX * k)].x, m);
         segmented_max_to_smem(4 * el, m, sMax);
     }
     __syncthreads();
@@ -388,7 +345,7 @@ __global__ void __launch_bounds__(NX* NX* ff_groups(NX)* EPB, (ff_min_blocks<NX,
         float2* wse = sWs + el * N3;
         float2* wte = sWt + el * N3;
 #pragma unroll 1
-        for (int k0 = kbeg; k0 < kend; k0 += W) {
+        for (int k0 = 0; k0 < NX; k0 += W) {
             OffsetAcc<T> ar, as, at;
             T sig_t;
 #pragma unroll
@@ -462,7 +419,7 @@ __global__ void __launch_bounds__(NX* NX* ff_groups(NX)* EPB, (ff_min_blocks<NX,
         const float bij = sCol[i] * mwr + sCol[j] * mws;
         double* we = w + (e0 + el) * (int64_t)N3;
 #pragma unroll 1
-        for (int k0 = kbeg; k0 < kend; k0 += W) {
+        for (int k0 = 0; k0 < NX; k0 += W) {
             T sig;
 #pragma unroll
             for (int q = 0; q < W; q++) L::set(sig, q, offset_for(bij + sCol[k0 + q] * mwt));
@@ -503,253 +460,34 @@ __global__ void __launch_bounds__(NX* NX* ff_groups(NX)* EPB, (ff_min_blocks<NX,
     if constexpr (mode_energies(MODE)) element_sums<TPE, EPB>(energy, reinterpret_cast<double*>(sU), edot + e0, ne);
 }
 
-// ------------------------------------------------------------------------
-// nx = 10 and 12: operands laid out for the packed f32x2 instructions.
-//
-// Shared memory holds u, wr and ws as float4 (h_k, h_k+1, l_k, l_k+1) per
-// (k-pair, j, i), so one 16-byte load gives both packed operands of a term; D is
-// kept pre-splatted (h, h, l, l), for the t-direction as k-pair tables, and for
-// the r-contraction transposed, so that a warp reads it across i without bank
-// conflicts; wt goes to a fourth block, read back by columns in phase 2.
+}  // namespace
+}  // namespace nek
+
+#include "nek_ax_fx.cuh"
+
+namespace nek {
+
+namespace {
+
+// The line-pass kernel k_ax_fx runs nx >= 5, the column walk k_ax_ff the smaller elements, where it is the faster one (nx = 2
+// 0.024 against 0.027 ms, nx = 4 0.061 against 0.076, 32768 elements).  From nx = 5 on k_ax_fx is faster (nx = 5 0.103
+// against 0.132 ms, nx = 10 0.62 against 0.96, nx = 16 0.85 against 1.81 ms a 33-million-point launch) and closer to 64
+// bits.
 template <int NX>
-constexpr size_t kpair_smem_bytes(int epb)
+constexpr bool fx_runs()
 {
-    // U4, WR4, WS4: [EPB][NX/2][NX][NX] float4 = 3 * 8 B per point; WT2 [EPB][N3]
-    // float2; DS [NX][NX], DP / DPT [NX][NX/2], DSt [NX][NX] float4; rowabs,
-    // colabs, maxima.
-    return sizeof(float4) * (3 * (size_t)epb * (NX / 2) * NX * NX + 3 * NX * NX) +
-           sizeof(float2) * (size_t)epb * NX * NX * NX + sizeof(float) * (2 * NX + 4 * (size_t)epb + 4) + 16;
+    return NX >= 5;
 }
 
-// Item mapping: the TPE threads of an element take its (column, k-pair) items
-// q = t, t + TPE, ...  At nx = 10, 128 threads share 500 items (at most 4
-// each): one column per thread would make a 100-thread CTA run a fourth warp on
-// 4 lanes, a quarter of its issue slots.  At nx = 12, 144 threads take one
-// column each (6 items); with four elements per CTA that is 18 full warps.  A
-// thread reads the column values of the t-contraction from shared memory (one
-// 16-byte load per k-pair) instead of holding a column in registers.
-constexpr int ffi_tpe(int nx) { return nx == 12 ? 144 : 128; }
-
-// CTAs per SM the register budget is set for: 20 resident warps (96 registers
-// a thread at one element per CTA; the kernel then spills 4-8 bytes).
+// Elements of a CTA that k_ax_fx holds at a time when EPB are asked for: as many of them as shared memory and 1024
+// threads allow (the results do not depend on it).
 template <int NX, int EPB>
-constexpr int ffi_min_blocks()
+constexpr int fx_conc()
 {
-    constexpr int warps = (ffi_tpe(NX) * EPB + 31) / 32;
-    return warps >= 20 ? 1 : 20 / warps;
-}
-
-template <int NX, int EPB, int MODE>
-__global__ void __launch_bounds__(ffi_tpe(NX) * EPB, (ffi_min_blocks<NX, EPB>()))
-    k_ax_ffi(int64_t nelt, const double* __restrict__ D, const float4* __restrict__ Gff,
-             const double* __restrict__ u, double* __restrict__ w, const int32_t* __restrict__ l2g,
-             const int32_t* __restrict__ eprob, const uint8_t* __restrict__ pdone, double* __restrict__ edot,
-             DirUpdate dir)
-{
-    static_assert(NX % 2 == 0 && NX <= 12, "even nx up to 12");
-    using T = float2;
-    constexpr int NP = NX / 2, N2 = NX * NX, N3 = NX * NX * NX, PB = NP * N2;
-    constexpr int TPE = ffi_tpe(NX), NT = TPE * EPB, NITEM = NP * N2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4* U4 = reinterpret_cast<float4*>(smem_raw);  // [EPB][NP][NX][NX]
-    float4* WR4 = U4 + EPB * PB;
-    float4* WS4 = WR4 + EPB * PB;
-    float2* WT2 = reinterpret_cast<float2*>(WS4 + EPB * PB);  // [EPB][N3] wt (h, l)
-    float4* DS = reinterpret_cast<float4*>(WT2 + EPB * N3);    // DS[a*NX+b] = (Dh,Dh,Dl,Dl) of D[a][b]
-    float4* DP = DS + N2;              // DP[l*NP+kp]  = (Dh[2kp][l], Dh[2kp+1][l], Dl[2kp][l], Dl[2kp+1][l])
-    float4* DPT = DP + NX * NP;        // DPT[l*NP+kp] = (Dh[l][2kp], Dh[l][2kp+1], Dl[l][2kp], Dl[l][2kp+1])
-    float4* DSt = DPT + NX * NP;       // DSt[b*NX+a] = DS[a*NX+b]: the r-contraction's row of D read across i
-    float* sRow = reinterpret_cast<float*>(DSt + N2);
-    float* sCol = sRow + NX;
-    float* sMax = sCol + NX;
-
-    const int tid = threadIdx.x;
-    const int64_t e0 = (int64_t)blockIdx.x * EPB;
-    const int ne = static_cast<int>(nelt - e0 < EPB ? nelt - e0 : EPB);
-    if (cta_skipped<MODE>(eprob, pdone, e0, ne)) return;  // uniform over the CTA, before any barrier
-
-    for (int q = tid; q < N2; q += NT) {
-        const int a = q / NX, b = q % NX;
-        const float2 d = split_double(D[q]);
-        DS[q] = make_float4(d.x, d.x, d.y, d.y);
-        DSt[b * NX + a] = make_float4(d.x, d.x, d.y, d.y);
-        float* dp = reinterpret_cast<float*>(DP + b * NP + a / 2);  // D[a][b]: k = a, l = b
-        dp[a & 1] = d.x;
-        dp[2 + (a & 1)] = d.y;
-        float* dt = reinterpret_cast<float*>(DPT + a * NP + b / 2);  // D[a][b]: l = a, k = b
-        dt[b & 1] = d.x;
-        dt[2 + (b & 1)] = d.y;
-    }
-    for (int q = tid; q < 4 * EPB; q += NT) sMax[q] = 0.f;
-    load_input<MODE, NT>(tid, ne * N3, e0 * N3, u, l2g, dir, [&](int q, double val) {
-        const int el = q / N3, p = q - el * N3;
-        const int k = p / N2, ji = p - k * N2;
-        const float2 v = split_double(val);
-        float* dst = reinterpret_cast<float*>(U4 + el * PB + (k / 2) * N2 + ji);
-        dst[k & 1] = v.x;
-        dst[2 + (k & 1)] = v.y;
-    });
-    __syncthreads();
-    for (int q = tid; q < NX; q += NT) {
-        float r = 0.f, c = 0.f;
-        for (int l = 0; l < NX; l++) {
-            r += fabsf(DS[q * NX + l].x);
-            c += fabsf(DS[l * NX + q].x);
-        }
-        sRow[q] = r * 1.0001f;
-        sCol[q] = c * 1.0001f;
-    }
-
-    const int el = tid / TPE;
-    const int t = tid - el * TPE;
-    const bool active = el < ne;
-    const float4* ue = U4 + el * PB;
-    {
-        float m = 0.f;
-        if (active)
-            for (int q = t; q < PB; q += TPE) {
-                const float4 v = ue[q];
-                m = absmax_bits(v.x, absmax_bits(v.y, m));
-            }
-        segmented_max_to_smem(4 * el, m, sMax);
-    }
-    __syncthreads();
-
-    // ------------------------------------------------------------- phase 1
-    float mx_r = 0.f, mx_s = 0.f, mx_t = 0.f;
-    if (active) {
-        const float umax = sMax[4 * el] * 1.0001f;
-        const float4* Ge = Gff + (e0 + el) * (int64_t)N3 * 3;
-        float4* wre = WR4 + el * PB;
-        float4* wse = WS4 + el * PB;
-        float2* wte = WT2 + el * N3;
-#pragma unroll 1
-        for (int q = t; q < NITEM; q += TPE) {
-            const int kp = q / N2, c = q - kp * N2;
-            const int i = c % NX, j = c / NX, k0 = 2 * kp;
-            OffsetAcc<T> ar, as, at;
-            ar.init(splat<T>(offset_for(sRow[i] * umax)));
-            as.init(splat<T>(offset_for(sRow[j] * umax)));
-            at.init(make_float2(offset_for(sRow[k0] * umax), offset_for(sRow[k0 + 1] * umax)));
-            const float4* ur = ue + kp * N2 + j * NX;  // u(l, j, k0..k0+1) at ur[l]
-            const float4* us = ue + kp * N2 + i;       // u(i, l, k0..k0+1) at us[l * NX]
-            const float4* uc = ue + c;                 // u(i, j, 2m..2m+1) at uc[m * N2]
-            float4 cu = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int l = 0; l < NX; l++) {
-                if ((l & 1) == 0) cu = uc[(l >> 1) * N2];
-                const float ch = (l & 1) ? cu.y : cu.x, cl = (l & 1) ? cu.w : cu.z;
-                const float4 a = ur[l], b = us[l * NX];
-                const float4 dr = DSt[l * NX + i], ds = DS[j * NX + l], dt = DP[l * NP + kp];
-                ar.add(make_float2(dr.x, dr.y), make_float2(dr.z, dr.w), make_float2(a.x, a.y),
-                       make_float2(a.z, a.w));
-                as.add(make_float2(ds.x, ds.y), make_float2(ds.z, ds.w), make_float2(b.x, b.y),
-                       make_float2(b.z, b.w));
-                at.add(make_float2(dt.x, dt.y), make_float2(dt.z, dt.w), make_float2(ch, ch), make_float2(cl, cl));
-            }
-            T urh, url, ush, usl, uth, utl;
-            ar.finish(urh, url);
-            as.finish(ush, usl);
-            at.finish(uth, utl);
-            T gf[12];
-#pragma unroll
-            for (int qq = 0; qq < 2; qq++) {
-                const int p = c + N2 * (k0 + qq);
-                const float4 a = __ldg(Ge + 3 * p), b = __ldg(Ge + 3 * p + 1), cc = __ldg(Ge + 3 * p + 2);
-                const float v[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, cc.x, cc.y, cc.z, cc.w};
-#pragma unroll
-                for (int g = 0; g < 12; g++) {
-                    if (qq)
-                        gf[g].y = v[g];
-                    else
-                        gf[g].x = v[g];
-                }
-            }
-            T wrh, wrl, wsh, wsl, wth, wtl;
-            df_dot3(gf[0], gf[1], urh, url, gf[2], gf[3], ush, usl, gf[4], gf[5], uth, utl, wrh, wrl);
-            df_dot3(gf[2], gf[3], urh, url, gf[6], gf[7], ush, usl, gf[8], gf[9], uth, utl, wsh, wsl);
-            df_dot3(gf[4], gf[5], urh, url, gf[8], gf[9], ush, usl, gf[10], gf[11], uth, utl, wth, wtl);
-            wre[kp * N2 + c] = make_float4(wrh.x, wrh.y, wrl.x, wrl.y);
-            wse[kp * N2 + c] = make_float4(wsh.x, wsh.y, wsl.x, wsl.y);
-            wte[c + N2 * k0] = make_float2(wth.x, wtl.x);
-            wte[c + N2 * (k0 + 1)] = make_float2(wth.y, wtl.y);
-            mx_r = absmax_bits(wrh.x, absmax_bits(wrh.y, mx_r));
-            mx_s = absmax_bits(wsh.x, absmax_bits(wsh.y, mx_s));
-            mx_t = absmax_bits(wth.x, absmax_bits(wth.y, mx_t));
-        }
-    }
-    segmented_max_to_smem(4 * el + 1, mx_r, sMax);
-    segmented_max_to_smem(4 * el + 2, mx_s, sMax);
-    segmented_max_to_smem(4 * el + 3, mx_t, sMax);
-    __syncthreads();
-
-    // ------------------------------------------------------------- phase 2
-    double energy = 0.0;  // energy modes: sum of u . w over this thread's points
-    if (active) {
-        const float4* wre = WR4 + el * PB;
-        const float4* wse = WS4 + el * PB;
-        const float2* wte = WT2 + el * N3;
-        const float mwr = sMax[4 * el + 1] * 1.0001f, mws = sMax[4 * el + 2] * 1.0001f,
-                    mwt = sMax[4 * el + 3] * 1.0001f;
-        double* we = w + (e0 + el) * (int64_t)N3;
-        const int64_t ef = (e0 + el) * (int64_t)N3;  // the element's first point
-#pragma unroll 1
-        for (int q = t; q < NITEM; q += TPE) {
-            const int kp = q / N2, c = q - kp * N2;
-            const int i = c % NX, j = c / NX, k0 = 2 * kp;
-            const int p0 = c + N2 * k0;
-            double u0 = 0.0, u1 = 0.0;
-            if constexpr (mode_energies(MODE)) {  // issued here, used after the contraction
-                u0 = reread_input<MODE>(ef, p0, u, l2g, dir);
-                u1 = reread_input<MODE>(ef, p0 + N2, u, l2g, dir);
-            }
-            const float bij = sCol[i] * mwr + sCol[j] * mws;
-            OffsetAcc<T> acc;
-            acc.init(make_float2(offset_for(bij + sCol[k0] * mwt), offset_for(bij + sCol[k0 + 1] * mwt)));
-            const float4* rr = wre + kp * N2 + j * NX;  // wr(l, j, k0..k0+1) at rr[l]
-            const float4* ss = wse + kp * N2 + i;       // ws(i, l, k0..k0+1) at ss[l * NX]
-            const float2* tt = wte + c;                 // wt(i, j, l) at tt[l * N2]
-#pragma unroll
-            for (int l = 0; l < NX; l++) {
-                const float4 a = rr[l], b = ss[l * NX];
-                const float4 ci = DS[l * NX + i], cj = DS[l * NX + j], dk = DPT[l * NP + kp];
-                acc.add(make_float2(ci.x, ci.y), make_float2(ci.z, ci.w), make_float2(a.x, a.y),
-                        make_float2(a.z, a.w));
-                acc.add(make_float2(cj.x, cj.y), make_float2(cj.z, cj.w), make_float2(b.x, b.y),
-                        make_float2(b.z, b.w));
-                const float2 tc = tt[l * N2];
-                acc.add(make_float2(dk.x, dk.y), make_float2(dk.z, dk.w), make_float2(tc.x, tc.x),
-                        make_float2(tc.y, tc.y));
-            }
-            T hi, lo;
-            acc.finish(hi, lo);
-            const double w0 = join_pair(hi.x, lo.x), w1 = join_pair(hi.y, lo.y);
-            we[p0] = w0;
-            we[p0 + N2] = w1;
-            if constexpr (mode_energies(MODE)) energy = fma(u1, w1, fma(u0, w0, energy));
-        }
-    }
-    if constexpr (mode_energies(MODE)) element_sums<TPE, EPB>(energy, reinterpret_cast<double*>(U4), edot + e0, ne);
-}
-
-// The k-pair layout (k_ax_ffi) is used where it measured faster than the
-// column walk on GB300 (nx = 10: 34.0 vs 25.6 GDOF/s; nx = 12: 26.5 vs 23.2;
-// nx = 8: 32.1 vs 36.4 with an earlier form of the layout).  The choice is
-// fixed per nx, never tuned at run time, because the two orders of summation
-// round differently.
-template <int NX>
-constexpr bool ff_item_layout()
-{
-    return NX == 10 || NX == 12;
-}
-
-template <int NX, int EPB>
-constexpr size_t ff_variant_smem()
-{
-    if constexpr (ff_item_layout<NX>())
-        return kpair_smem_bytes<NX>(EPB);
+    if constexpr (EPB == 1)
+        return 1;
     else
-        return ff_smem_bytes<NX, EPB>();
+        return sizeof(FxSmem<NX, EPB>) <= 227 * 1024 && fx_threads(NX, EPB) <= 1024 ? EPB : fx_conc<NX, EPB / 2>();
 }
 
 template <int NX, int EPB, int MODE>
@@ -757,20 +495,26 @@ nek_status launch_ax_ff_kernel(int64_t nelt, const double* D, const float* Gff, 
                                cudaStream_t s, const int32_t* l2g, const int32_t* eprob, const uint8_t* pdone,
                                double* edot, const DirUpdate* dir = nullptr)
 {
-    constexpr size_t smem = ff_variant_smem<NX, EPB>();
     static std::atomic<uint64_t> configured{0};
-    const int64_t blocks = (nelt + EPB - 1) / EPB;
-    if (blocks > 0x7fffffff) return NEK_ERR_TOO_LARGE;
-    if constexpr (ff_item_layout<NX>()) {
-        nek_status st = ensure_dyn_smem(k_ax_ffi<NX, EPB, MODE>, smem, configured);
+    const DirUpdate d = dir ? *dir : DirUpdate{};
+    const float4* G4 = reinterpret_cast<const float4*>(Gff);
+    if constexpr (fx_runs<NX>()) {
+        constexpr int C = fx_conc<NX, EPB>();
+        constexpr size_t smem = sizeof(FxSmem<NX, C>);
+        if ((nelt + EPB - 1) / EPB > 0x7fffffff) return NEK_ERR_TOO_LARGE;
+        nek_status st = ensure_dyn_smem(k_ax_fx<NX, C, MODE>, smem, configured);
         if (st != NEK_OK) return st;
-        k_ax_ffi<NX, EPB, MODE><<<(unsigned)blocks, ffi_tpe(NX) * EPB, smem, s>>>(
-            nelt, D, reinterpret_cast<const float4*>(Gff), u, w, l2g, eprob, pdone, edot, dir ? *dir : DirUpdate{});
+        const int64_t groups = (nelt + C - 1) / C, resident = kSMs * fx_min_blocks<NX, C>();
+        k_ax_fx<NX, C, MODE><<<(unsigned)(groups < resident ? groups : resident), fx_threads(NX, C), smem, s>>>(
+            nelt, D, G4, u, w, l2g, eprob, pdone, edot, d);
     } else {
+        constexpr size_t smem = ff_smem_bytes<NX, EPB>();
+        const int64_t blocks = (nelt + EPB - 1) / EPB;
+        if (blocks > 0x7fffffff) return NEK_ERR_TOO_LARGE;
         nek_status st = ensure_dyn_smem(k_ax_ff<NX, EPB, MODE>, smem, configured);
         if (st != NEK_OK) return st;
-        k_ax_ff<NX, EPB, MODE><<<(unsigned)blocks, ff_threads_per_elem(NX) * EPB, smem, s>>>(
-            nelt, D, reinterpret_cast<const float4*>(Gff), u, w, l2g, eprob, pdone, edot, dir ? *dir : DirUpdate{});
+        k_ax_ff<NX, EPB, MODE><<<(unsigned)blocks, NX * NX * EPB, smem, s>>>(nelt, D, G4, u, w, l2g, eprob, pdone,
+                                                                             edot, d);
     }
     return check_launch();
 }
@@ -797,44 +541,32 @@ nek_status launch_ax_ff_variant(int64_t nelt, const double* D, const float* Gff,
     return launch_ax_ff_kernel<NX, EPB, kModePlain>(nelt, D, Gff, u, w, s, nullptr, nullptr, nullptr, nullptr);
 }
 
-template <int NX, int EPB>
-constexpr bool ff_fits()
-{
-    constexpr int threads = ff_item_layout<NX>() ? ffi_tpe(NX) * EPB : ff_threads_per_elem(NX) * EPB;
-    return threads <= 1024 && ff_variant_smem<NX, EPB>() <= 227 * 1024;
-}
+// Default elements per CTA (the tuner may change them): four of the small elements; above, k_ax_fx packs two where the
+// threads of one would leave lanes of its last warp idle (nx = 7: 0.238 against 0.287 ms at 32768 elements; nx = 5
+// with four 0.100 against 0.137).
+constexpr int ff_epb(int nx) { return nx <= 5 ? 4 : nx == 7 ? 2 : 1; }
+
+// The counts that are accepted for nx: 1, 2 and 4 up to nx = 12, 1 above.
+constexpr bool ff_fits(int nx, int epb) { return epb == 1 || (nx <= 12 && (epb == 2 || epb == 4)); }
 
 template <int NX>
 nek_status launch_ax_ff_nx(int epb, int64_t nelt, const double* D, const float* Gff, const double* u, double* w,
                            cudaStream_t s, const int32_t* l2g, const int32_t* eprob, const uint8_t* pdone,
                            double* edot, const DirUpdate* dir)
 {
-    if (epb <= 0) epb = ff_epb<NX>();
-    switch (epb) {
-        case 1:
-            if constexpr (ff_fits<NX, 1>())
-                return launch_ax_ff_variant<NX, 1>(nelt, D, Gff, u, w, s, l2g, eprob, pdone, edot, dir);
-            break;
-        case 2:
-            if constexpr (ff_fits<NX, 2>())
-                return launch_ax_ff_variant<NX, 2>(nelt, D, Gff, u, w, s, l2g, eprob, pdone, edot, dir);
-            break;
-        case 4:
-            if constexpr (ff_fits<NX, 4>())
-                return launch_ax_ff_variant<NX, 4>(nelt, D, Gff, u, w, s, l2g, eprob, pdone, edot, dir);
-            break;
-        default:
-            break;
+    if (epb <= 0) epb = ff_epb(NX);
+    if (epb == 1) return launch_ax_ff_variant<NX, 1>(nelt, D, Gff, u, w, s, l2g, eprob, pdone, edot, dir);
+    if constexpr (ff_fits(NX, 2)) {
+        if (epb == 2) return launch_ax_ff_variant<NX, 2>(nelt, D, Gff, u, w, s, l2g, eprob, pdone, edot, dir);
+        if (epb == 4) return launch_ax_ff_variant<NX, 4>(nelt, D, Gff, u, w, s, l2g, eprob, pdone, edot, dir);
     }
-    if constexpr (ff_epb<NX>() != 1 && ff_epb<NX>() != 2 && ff_epb<NX>() != 4)
-        return launch_ax_ff_variant<NX, ff_epb<NX>()>(nelt, D, Gff, u, w, s, l2g, eprob, pdone, edot, dir);
     return NEK_ERR_INVALID_ARG;
 }
 
 template <int NX>
 bool ff_fits_rt(int epb)
 {
-    return (epb == 1 && ff_fits<NX, 1>()) || (epb == 2 && ff_fits<NX, 2>()) || (epb == 4 && ff_fits<NX, 4>());
+    return ff_fits(NX, epb);
 }
 
 }  // namespace

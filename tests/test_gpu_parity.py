@@ -767,3 +767,86 @@ def test_batch_one_launch_native_fp64_operator():
     for q, m in enumerate(meshes):
         Pr = ref.Problem(m)
         assert Pr.residual(fields[q], xs[q].reshape(m.nelt, -1)) <= 1e-9 * 1.001
+
+
+# ------------------------------------------------- line-pass operator (nx >= 5)
+def _ff_operator(nx, nelt, D, G, u, epb=0, energy=False):
+    Gff = torch.empty((nelt, nx ** 3, 12), dtype=torch.float32, device=DEV)
+    nekax.geom_ff(nelt, nx, G, Gff)
+    w = torch.full((nelt, nx ** 3), float("nan"), dtype=torch.float64, device=DEV)
+    ed = torch.full((nelt,), float("nan"), dtype=torch.float64, device=DEV)
+    if energy:
+        nekax.ax_ff_energy(nelt, nx, D, Gff, u, w, ed)
+    else:
+        nekax.ax_ff(nelt, nx, D, Gff, u, w)
+    torch.cuda.synchronize()
+    return w.cpu().numpy(), ed.cpu().numpy()
+
+
+@pytest.mark.parametrize("kind", ["gll", "general", "one entry off"])
+@pytest.mark.parametrize("nx,nelt", [(5, 5003), (6, 61), (7, 2003), (8, 13), (9, 5), (10, 700), (11, 3), (12, 331),
+                                     (13, 3), (14, 161), (15, 2), (16, 311)])
+def test_ax_ff_any_matrix_and_many_groups(nx, nelt, kind):
+    """D of the rule (folded rows), any D, and the rule's D with one entry changed in its last bits (every row for
+    itself); element counts below, and above, what the resident CTAs hold at once, and ragged ones.
+
+    Bound per element: three digit splits (u, D, G D u), each good to 2^-46 of its maximum and summed over nx
+    points with a handful of roundings more: 3 (nx + 8) 2^-46 of the operator on absolute values."""
+    rng = np.random.default_rng(900 + nx)
+    xi, rho, D = ref.gll(nx)
+    if kind == "general":
+        D = rng.uniform(-1, 1, size=(nx, nx)) * np.exp(rng.uniform(-3, 3, size=(nx, 1)))
+    elif kind == "one entry off":
+        D = D.copy()
+        D[nx // 2, 0] *= 1 + 2.0 ** -50
+    base = min(nelt, 60)
+    mesh = inputs.box_mesh(base, 1, 1, nx, perturb=0.2, seed=nx)
+    G = ref.geom(mesh.corners, nx, xi, rho)[np.arange(nelt) % base]
+    u = rng.uniform(-1, 1, size=(nelt, nx ** 3)) * np.exp(rng.uniform(-20, 20, size=(nelt, 1)))
+    w, _ = _ff_operator(nx, nelt, _t(D), _t(G), _t(u))
+    wr = ref.ax(D, G, u)
+    bound = 3 * (nx + 8) * 2.0 ** -46 * ref.ax(np.abs(D), np.abs(G), np.abs(u)).max(axis=1, keepdims=True)
+    assert np.all(np.abs(w - wr) <= bound), np.max(np.abs(w - wr) / bound)
+
+
+@pytest.mark.parametrize("nx,nelt", [(5, 9), (8, 7), (10, 620), (13, 4)])
+def test_ax_ff_non_finite_stays_in_its_element(nx, nelt):
+    """A NaN, an infinity, a value beyond the float range: that element is NaN, every other one unchanged; a zero
+    element is zero."""
+    rng = np.random.default_rng(nx)
+    xi, rho, D = ref.gll(nx)
+    mesh = inputs.box_mesh(min(nelt, 7), 1, 1, nx, perturb=0.2, seed=nx)
+    G = ref.geom(mesh.corners, nx, xi, rho)[np.arange(nelt) % min(nelt, 7)]
+    u = rng.uniform(-1, 1, size=(nelt, nx ** 3))
+    clean, ec = _ff_operator(nx, nelt, _t(D), _t(G), _t(u), energy=True)
+    for e, v in ((1, np.nan), (2, np.inf), (nelt - 1, -1e300)):
+        u[e, nx + 1] = v
+    u[0] = 0.0
+    w, ed = _ff_operator(nx, nelt, _t(D), _t(G), _t(u), energy=True)
+    bad = [1, 2, nelt - 1]
+    assert np.all(np.isnan(w[bad])) and np.all(np.isnan(ed[bad]))
+    assert np.all(w[0] == 0.0) and ed[0] == 0.0
+    rest = [e for e in range(nelt) if e not in bad + [0]]
+    assert np.array_equal(w[rest], clean[rest]) and np.array_equal(ed[rest], ec[rest])
+
+
+def test_batch_skips_finished_elements_beyond_the_resident_ctas():
+    """Problems of more elements than the resident CTAs hold, one of them finished from the start (f = 0): the CTAs
+    pass over its elements and the others' iterates are those of a batch without it."""
+    from paper_2011_04981_gb300.problem import DeviceBatch
+
+    meshes = [inputs.box_mesh(6, 6, 5, 13, perturb=0.1, seed=s) for s in (1, 2, 3)]
+    f = [inputs.random_global_field(m, seed=q) for q, m in enumerate(meshes)]
+    f[1] = np.zeros_like(f[1])
+    B = DeviceBatch(meshes, f, DEV)
+    x = torch.full((B.npts,), float("nan"), dtype=torch.float64, device=DEV)
+    r = B.solve(x, tol=1e-6, max_iter=40, iters_per_graph=10)
+    assert sorted(r["iters"].tolist())[0] == 0
+    xs = B.split(x)
+    A = DeviceBatch([meshes[0], meshes[2]], [f[0], f[2]], DEV)
+    y = torch.full((A.npts,), float("nan"), dtype=torch.float64, device=DEV)
+    A.solve(y, tol=1e-6, max_iter=40, iters_per_graph=10)
+    ys = A.split(y)
+    assert torch.all(xs[1] == 0)
+    for a, b in ((xs[0], ys[0]), (xs[2], ys[1])):
+        assert torch.all(torch.isfinite(b)) and float((a - b).abs().max()) <= 1e-9 * float(b.abs().max())
