@@ -23,10 +23,10 @@
 // built once, the next element's input is copied to shared memory (cp.async, in the place of the split
 // form) under the current one's second half, and the element's G is fetched into L2 while phase 1 runs.
 //
-// What bounds it (nx = 10, 32768 elements, ncu): no unit is saturated; issue 52 %, shared-memory data path 61 %, FMA pipes 36 %,
-// and 4.8 warps a scheduler wait on fixed latencies (1.4 cycles an instruction), global loads (1.4), shared loads (0.8) and
-// barriers (0.9).  0.62 ms = 53 GDOF/s = 0.50 of the measured HBM copy rate at 64 B/point (float-float
-// item kernel before: 0.96 ms); with the solve's direction update 0.82 ms = 0.61 of it at 104 B/point (1.04 ms before).
+// What bounds it (nx = 10, 32768 elements, ncu): no unit is saturated; issue 52 %, shared-memory data path 61 %, FMA
+// pipes 36 %; the 4.8 warps a scheduler wait on fixed latencies, global loads, shared loads and barriers in about equal
+// parts.  0.62 ms = 53 GDOF/s = 0.50 of the measured HBM copy rate at 64 B/point (float-float item kernel before: 0.96
+// ms); with the solve's direction update 0.82 ms = 0.61 of it at 104 B/point (1.04 ms before).
 #pragma once
 
 #include <type_traits>

@@ -1,28 +1,33 @@
 // Learned-preconditioner inference on the 5th-generation tensor cores (tcgen05):
 // BF16 operands in shared memory, FP32 accumulators in tensor memory (TMEM).
 //
-// Each 3x3x3 convolution of the per-element network is an implicit GEMM with
-// M = output points, K = 16 input channels of one tap, N = 16 output channels,
-// accumulated over the 27 taps.  The activations of one element are kept in
-// shared memory on a zero-padded 10 x 10 x 10 grid of 16-byte rows (8 BF16
-// channels per row; the 16 channels are two such arrays, the two K halves of
-// the MMA's A operand):
-//     row (i', j', k') at byte 16 * (10 * L + i'),  L = 10 k' + j' + 1,
-// i' = i + 1 etc., plus one guard line (L = 0 and L = 101) at each end.  An M = 128
-// tile covers 16 consecutive "padded lines" L_out = 10 k + j' of the output
-// (8 points each, the i direction); for tap (di, dj, dk) the A rows of those 16
-// lines are 16 lines of the grid at the uniform line stride, shifted by
-// 10 (1 + dk) + dj lines and 1 + di rows, so every tap is one descriptor with the
-// same strides (SBO = 160 B between 8-row groups, LBO = the K-half array size).
-// The 80 padded output lines (k = 0..7, j' = 0..9) make 5 tiles; rows on the
-// padding lines j' = 0, 9 compute garbage from in-range addresses and are
-// dropped by the epilogue.  Per element and layer: 5 x 27 MMAs of
-// 128 x 16 x 16 issued by one thread, committed to an mbarrier.
+// Each 3x3x3 convolution of the per-element network is an implicit GEMM whose rows are the lines of points along i.
+// Two elements at a time make one M = 128 tile: row m = 8 (2 k + e) + j is line (j, k) of element e.  The
+// activations of point i of every line lie together,
+//     point i, K half h, padded plane kk = k + 1, element e, padded line jj = j + 1:
+//     16-byte row (8 BF16 channels) at 5184 i + 2592 h + 144 (2 kk + e) + 16 jj,
+// on a zero-padded grid of (jj, kk) whose last zero line and plane are the next one's first, so the A operand of a
+// tap (dj, dk) is one descriptor with the strides LBO = 2592 B, SBO = 144 B, shifted by
+// 16 (1 + dj) + 288 (1 + dk).  The three taps along i go to N: the MMA of input point i multiplies by a 16 x 48
+// operand (di = +1, 0, -1) into the TMEM columns of the output points i - 1, i and i + 1 (16 channels each, 128 columns
+// a tile): 78 MMAs a layer and two elements, where one MMA per tap takes 270 of N = 16.  An MMA of so few columns takes the time to read its 4 KB of A from shared memory, so the reads are
+// what counts.  Every output still sums its 27 taps in the order (dk, dj, di), one MMA each: the sums are
+// bit-identical to those of one MMA per tap.  The first (dj, dk) overwrites: the point i + 1 that an MMA reaches
+// first is a 16-column MMA of its own there.
 //
-// The epilogue reads each thread's TMEM lane (one output row) with tcgen05.ld,
-// adds the bias, applies GELU in FP32, rounds to BF16 and writes the row back
-// into the same grid (the next layer's input; every MMA of the layer has
+// A CTA has four groups of eight warps, each with its own tile (41 KB of activations, 128 TMEM columns) and
+// mbarrier; the weights (41 KB) are shared.  A group is a chain of MMAs, wait and epilogue per layer; the groups'
+// chains overlap.  One CTA per SM, persistent over pairs of elements.
+//
+// The epilogue reads each thread's TMEM lane (one line) with tcgen05.ld, adds the bias, applies GELU in FP32,
+// rounds to BF16 and writes the rows back in place (the next layer's input; every MMA of the layer has
 // completed by then).  The last layer writes z = y * scale * c in FP64.
+//
+// What bounds it (13 824 elements, 362 us against 975 before; 322 TFLOP/s of useful work): the MMAs alone, with
+// the GELUs left out, take 263 us, about 50 cycles each for the 42 shared-memory wavefronts of their operands; the GELUs alone
+// (25 instructions, ten of them on the half-rate ALU pipe) about 200 us of issue.  Three groups of four warps took
+// 500 us, three of eight 440, four of eight 418, and 362 once one elected thread issues all MMAs with operands in
+// uniform registers (20 instructions an MMA before, which the issuing warp did not get through between the GELUs).
 //
 // Numerics are those of nek_net_apply_bf16's contract: BF16 weights, the input
 // and both hidden activations rounded to BF16 (nearest even) before each
@@ -30,12 +35,13 @@
 //
 // Every wait on the mbarrier is bounded (~2 s of global time).  A wait that runs
 // out sets a device flag (read by nek_fcg_solve_trunc, which returns
-// NEK_ERR_TIMEOUT), writes NaN into the element's output (so the solve that uses
-// it stops on a non-finite value), waits once more, frees the CTA's TMEM and
+// NEK_ERR_TIMEOUT), writes NaN into the tile's outputs (so the solve that uses
+// it stops on a non-finite value), waits once more and ends its group; the CTA then frees its TMEM and
 // returns.
 #include <cuda_bf16.h>
 
 #include "nek_internal.h"
+#include "nek_tc5.cuh"
 
 namespace nek {
 
@@ -45,226 +51,228 @@ constexpr int NP = 512, CIN = 2, CH = 16;
 constexpr int NPARAM_TC5 = CH * CIN * 27 + CH + CH * CH * 27 + CH + CH * 27 + 1;
 constexpr int OW1 = 0, OB1 = OW1 + CH * CIN * 27, OW2 = OB1 + CH, OB2 = OW2 + CH * CH * 27, OW3 = OB2 + CH,
               OB3 = OW3 + CH * 27;
-constexpr int NT5 = 128;            // 4 warps: one per 32-lane TMEM sub-partition
-constexpr int kLines = 102;         // 100 grid lines + 2 guard lines
-constexpr int kHalfBytes = kLines * 10 * 16;  // one K half of the activation grid: 16320 B
-constexpr int kTapBytes = 512;      // B operand of one tap: 16 rows (n) x 16 channels (k), two K halves
-constexpr int kTiles = 5;           // 80 padded output lines / 16
-constexpr uint32_t kTmemCols = 128; // 5 tiles x 16 columns, rounded up to a power of two
-constexpr long long kWaitNs = 2000000000LL;  // default bound of every mbarrier wait
-
-// 32-bit instruction descriptor of tcgen05.mma kind::f16: D FP32 (bits 4-5 = 1),
-// A and B BF16 (bits 7-9 and 10-12 = 1), both K-major (bits 15, 16 = 0),
-// N >> 3 in bits 17-22, M >> 4 in bits 24-28.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr int kGroups = 4, kGroupThreads = 256;  // eight warps: two per 32-lane TMEM sub-partition
+constexpr int kLine8 = 144;                      // bytes between the two elements' groups of 8 lines (and a zero one)
+constexpr int kPlane2 = 2 * kLine8;              // between planes
+constexpr int kHalf = 9 * kPlane2;               // K half (8 channels) of one point's activations; the plane after it is the
+constexpr int kPoint = 2 * kHalf;                // next one's zero plane
+constexpr int kTile = 8 * kPoint + kPlane2 + 16;
+constexpr int kTapHalf = 48 * 16, kTap = 2 * kTapHalf;  // B operand of one (dj, dk): [K half][n][8 channels]
+constexpr uint32_t kHint = 1000;  // ns that a wait may sleep at a time
+constexpr uint32_t kTmemCols = 128 * kGroups;
+constexpr long long kWaitNs = 2000000000LL;             // default bound of every mbarrier wait
 
 struct __align__(128) Tc5Smem {
-    __nv_bfloat16 act[2 * kLines * 10 * 8];  // [K half][line][row][8 channels]
-    __nv_bfloat16 w[3 * 27 * 2 * 16 * 8];     // [layer][tap][K half][n][8 channels]
+    unsigned char w[3][9][kTap];
+    unsigned char act[kGroups][kTile];
     float b1[16], b2[16], b3[4];
-    unsigned long long mbar;
+    unsigned long long mbar[kGroups];
     uint32_t tmem_base;
 };
 
 __device__ int g_net_tc5_timeout = 0;  // set by a bounded wait that ran out
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
 __device__ __forceinline__ float gelu5(float v) { return 0.5f * v * (1.f + erff(v * 0.70710678118654752f)); }
 
-// Shared-memory matrix descriptor (no swizzle): start address, LBO (K direction),
-// SBO (M/N direction, 8-row groups), all >> 4; the fixed value 1 in bits 46-48.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
+// Barrier of one group (ids 1 ..), and the same with the disjunction of a predicate.
+__device__ __forceinline__ void group_sync(int g)
 {
-    uint64_t d = (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(g + 1), "r"(kGroupThreads) : "memory");
 }
-
-__device__ __forceinline__ void mma_bf16_tmem(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t accumulate)
+__device__ __forceinline__ bool group_or(int g, bool v)
 {
+    uint32_t r;
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(kIdesc), "r"(accumulate));
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %3, 0;\n\t"
+        "barrier.cta.red.or.pred q, %1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(r)
+        : "r"(g + 1), "r"(kGroupThreads), "r"((uint32_t)v)
+        : "memory");
+    return r != 0;
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t mbar)
+// Channel 0 of four consecutive points of the lane (columns 0, 16, 32, 48 from t), loads and wait in one statement.
+__device__ __forceinline__ void tmem_ld_points(uint32_t t, float (&y)[4])
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-                 : "memory");
+    uint32_t r[4];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%4];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%1}, [%5];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%2}, [%6];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%3}, [%7];\n\t"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3])
+        : "r"(t), "r"(t + 16), "r"(t + 32), "r"(t + 48)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 4; i++) y[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ long long global_ns()
+// The MMAs of one layer (one elected thread): every tap of every point into the tile's 128 columns.
+__device__ __forceinline__ void layer_mmas(uint32_t d, uint64_t a0, uint64_t b0)
 {
-    long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Wait for the mbarrier phase with parity `parity`; false if it did not complete
-// within kWaitNs.  Each try may suspend the thread (up to the hint, 20 us) until
-// the phase completes, so waiting threads do not take issue slots from the
-// other CTAs on the SM; the clock is read every 64 tries.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar, uint32_t parity, long long wait_ns)
-{
-    const long long t0 = global_ns();
-    for (int tries = 1;; tries++) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred P1;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2, %3;\n\t"
-            "selp.b32 %0, 1, 0, P1;\n\t}\n"
-            : "=r"(done)
-            : "r"(mbar), "r"(parity), "r"(20000)
-            : "memory");
-        if (done) return true;
-        if ((tries & 63) == 0 && global_ns() - t0 > wait_ns) return false;
+    constexpr uint32_t i16 = tc5::idesc_bf16_f32(128, 16), i32 = tc5::idesc_bf16_f32(128, 32),
+                       i48 = tc5::idesc_bf16_f32(128, 48);
+    // the first (dj, dk): point i reaches output i + 1 for the first time
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const uint64_t a = a0 + (uint64_t)(i * (kPoint >> 4));
+        if (i == 0)
+            tc5::mma_bf16(d, a, b0 + 16, i32, 0u);  // outputs 0 and 1
+        else {
+            tc5::mma_bf16(d + 16u * (i - 1), a, b0, i32, 1u);  // outputs i - 1 and i
+            if (i < 7) tc5::mma_bf16(d + 16u * (i + 1), a, b0 + 32, i16, 0u);
+        }
+    }
+#pragma unroll 1
+    for (int q = 1; q < 9; q++) {
+        const uint64_t aq = a0 + (uint64_t)((q / 3) * (kPlane2 >> 4) + q % 3), b = b0 + (uint64_t)(q * (kTap >> 4));
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const uint64_t a = aq + (uint64_t)(i * (kPoint >> 4));
+            if (i == 0)
+                tc5::mma_bf16(d, a, b + 16, i32, 1u);
+            else
+                tc5::mma_bf16(d + 16u * (i - 1), a, b, i < 7 ? i48 : i32, 1u);
+        }
     }
 }
 
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// 16 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int q = 0; q < 16; q++) v[q] = __uint_as_float(r[q]);
-}
-
-// Byte offset of grid row (i', j', k') in one K half.
-__device__ __forceinline__ int grid_row(int ip, int jp, int kp) { return 16 * (10 * (10 * kp + jp + 1) + ip); }
-
-// arrivals: arrivals the mbarrier expects per phase (1: the commit of the MMAs;
+// arrivals: arrivals the mbarriers expect per phase (1: the commit of the MMAs;
 // the self-test passes 2, which no phase ever gets, so every wait runs out).
-__global__ void __launch_bounds__(NT5, 3) k_net_apply_tc5(int64_t nelt, const float* __restrict__ theta,
-                                                         const float* __restrict__ xin,
-                                                         const float* __restrict__ scale,
-                                                         const double* __restrict__ c, double* __restrict__ z,
-                                                         long long wait_ns, int arrivals)
+__global__ void __launch_bounds__(kGroups* kGroupThreads, 1)
+    k_net_apply_tc5(int64_t nelt, const float* __restrict__ theta, const float* __restrict__ xin,
+                    const float* __restrict__ scale, const double* __restrict__ c, double* __restrict__ z,
+                    long long wait_ns, int arrivals)
 {
     extern __shared__ __align__(128) unsigned char raw5[];
     Tc5Smem& S = *reinterpret_cast<Tc5Smem*>(raw5);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned char* act = reinterpret_cast<unsigned char*>(S.act);
+    constexpr int NT = kGroups * kGroupThreads;
+    const int tid = threadIdx.x, warp = tid >> 5, grp = tid / kGroupThreads;
 
-    // ---- set-up: weights as BF16 B operands, zero grid, biases, mbarrier, TMEM
-    for (int q = tid; q < 3 * 27 * 2 * 16 * 8; q += NT5) {
-        const int k8 = q & 7, n = (q >> 3) & 15, h = (q >> 7) & 1, t = (q >> 8) % 27, l = (q >> 8) / 27;
-        const int ch = 8 * h + k8;
+    // ---- set-up: weights as BF16 B operands, zero grids, biases, mbarriers, TMEM
+    for (int q = tid; q < 3 * 9 * 2 * 48 * 8; q += NT) {
+        const int k8 = q & 7, n = (q >> 3) % 48, h = (q / (8 * 48)) & 1, t9 = (q / (16 * 48)) % 9, l = q / (16 * 48 * 9);
+        const int ch = 8 * h + k8, o = n & 15, t = 3 * t9 + 2 - (n >> 4);  // n = 0..15: di = +1
         float v = 0.f;
-        if (l == 0 && ch < CIN) v = theta[OW1 + (n * CIN + ch) * 27 + t];
-        if (l == 1) v = theta[OW2 + (n * CH + ch) * 27 + t];
-        if (l == 2 && n == 0) v = theta[OW3 + ch * 27 + t];
-        S.w[q] = __float2bfloat16_rn(v);
+        if (l == 0 && ch < CIN) v = theta[OW1 + (o * CIN + ch) * 27 + t];
+        if (l == 1) v = theta[OW2 + (o * CH + ch) * 27 + t];
+        if (l == 2 && o == 0) v = theta[OW3 + ch * 27 + t];
+        reinterpret_cast<__nv_bfloat16*>(S.w)[q] = __float2bfloat16_rn(v);
     }
-    for (int q = tid; q < 2 * kLines * 10 * 8 / 8; q += NT5) reinterpret_cast<uint4*>(S.act)[q] = make_uint4(0, 0, 0, 0);
+    for (int q = tid; q < kGroups * kTile / 16; q += NT) reinterpret_cast<uint4*>(S.act)[q] = make_uint4(0, 0, 0, 0);
     if (tid < CH) {
         S.b1[tid] = __bfloat162float(__float2bfloat16_rn(theta[OB1 + tid]));
         S.b2[tid] = __bfloat162float(__float2bfloat16_rn(theta[OB2 + tid]));
     }
     if (tid == 0) {
         S.b3[0] = __bfloat162float(__float2bfloat16_rn(theta[OB3]));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&S.mbar)), "r"(arrivals) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int g = 0; g < kGroups; g++) tc5::mbar_init(tc5::smem_u32(&S.mbar[g]), arrivals);
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)),
-                     "r"(kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    fence_async_smem();
-    tc_fence_before();
+    if (warp == 0) tc5::tmem_alloc(&S.tmem_base, kTmemCols);
+    tc5::fence_async_smem();
+    tc5::fence_before();
     __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = S.tmem_base;
-    const uint32_t mbar = smem_u32(&S.mbar);
-    const uint32_t act_base = smem_u32(S.act), w_base = smem_u32(S.w);
-    // descriptors of the grid's first row (LBO = one K half, SBO = one line) and of layer 0, tap 0
-    const uint64_t a_desc0 = smem_desc(act_base, kHalfBytes, 160);
-    const uint64_t b_desc0 = smem_desc(w_base, 256, 128);
+    tc5::fence_after();
+    // warp-uniform by construction (broadcast from lane 0), so that the MMAs' operands live in uniform registers
+    const int ugrp = __shfl_sync(0xffffffffu, grp, 0);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, S.tmem_base, 0), d_tile = tmem + 128u * (uint32_t)ugrp;
+    const uint32_t mbar = tc5::smem_u32(&S.mbar[ugrp]);
+    unsigned char* act = S.act[ugrp];
+    const uint64_t a0 = tc5::smem_desc(tc5::smem_u32(act), kHalf, kLine8);  // tap (dj, dk) = (-1, -1) of point 0
+    const uint64_t b0 = tc5::smem_desc(tc5::smem_u32(S.w), kTapHalf, 128);
     uint32_t parity = 0;
-    // This thread's TMEM lane: row m of every tile (warp w owns lanes 32 w .. 32 w + 31).
-    const int m = 32 * warp + lane;
-    const uint32_t lane_addr = tmem + ((uint32_t)(32 * warp) << 16);
-    bool failed = false;  // uniform across the CTA (decided by __syncthreads_or)
+    // this thread's line (its TMEM lane m: element e of the pair, j, k), the four points i0 .. i0 + 3 of it, and the
+    // place of its rows at point i0
+    const int m = tid & 127, e = (m >> 3) & 1, j = m & 7, k = m >> 4, i0 = (tid >> 5) & 4;
+    const uint32_t lane_addr = d_tile + ((uint32_t)(32 * (warp & 3)) << 16) + 16u * (uint32_t)i0;
+    unsigned char* rows = act + kPoint * i0 + kPlane2 * (k + 1) + kLine8 * e + 16 * (j + 1);
+    const bool vec = (reinterpret_cast<uintptr_t>(xin) & 15) == 0;
+    const bool vecz = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(c)) & 15) == 0;
 
-    for (int64_t e = blockIdx.x; e < nelt; e += gridDim.x) {
-        // input: channels 0, 1 of the interior rows (rounded to BF16), channels 2..15 zero
-        for (int p = tid; p < NP; p += NT5) {
-            const int i = p & 7, j = (p >> 3) & 7, k = p >> 6;
-            const __nv_bfloat162 x01 = __floats2bfloat162_rn(xin[(e * CIN + 0) * NP + p], xin[(e * CIN + 1) * NP + p]);
-            const int off = grid_row(i + 1, j + 1, k + 1);
-            uint4 h0 = make_uint4(*reinterpret_cast<const uint32_t*>(&x01), 0u, 0u, 0u);
-            *reinterpret_cast<uint4*>(act + off) = h0;
-            *reinterpret_cast<uint4*>(act + kHalfBytes + off) = make_uint4(0, 0, 0, 0);
-        }
-        const double sc = (double)scale[e];
-        for (int layer = 0; layer < 3; layer++) {
-            fence_async_smem();  // the grid's rows, written by this CTA's threads, are read by the tensor core
-            tc_fence_before();
-            __syncthreads();
-            tc_fence_after();
-            if (warp == 0) {
-                if (lane == 0) {
-                    // descriptors advance by (byte offset >> 4) in their start-address field
-                    const uint64_t b_layer = b_desc0 + (uint64_t)((layer * 27 * kTapBytes) >> 4);
-#pragma unroll 1
-                    for (int tile = 0; tile < kTiles; tile++) {
-                        const uint64_t a_tile = a_desc0 + (uint64_t)(16 * tile * 10);  // 16 lines of 160 B
-                        const uint32_t d = tmem + 16u * (uint32_t)tile;
+    const int64_t npair = (nelt + 1) / 2, step = (int64_t)gridDim.x * kGroups;
+    // the points' two input channels (zero where the pair has no second element)
+    float x[2][4];
+    auto load_line = [&](int64_t pair) {
+        const int64_t el = 2 * pair + e;
 #pragma unroll
-                        for (int t = 0; t < 27; t++) {
-                            const int dk = t / 9 - 1, dj = (t / 3) % 3 - 1, di = t % 3 - 1;
-                            // first row of the tile's A rows: line 11 + 10 dk + dj, row 1 + di (in 16-byte units)
-                            const int a_off = 10 * (11 + 10 * dk + dj) + 1 + di;
-                            mma_bf16_tmem(d, a_tile + (uint64_t)a_off, b_layer + (uint64_t)(t * (kTapBytes >> 4)),
-                                          t > 0 ? 1u : 0u);
-                        }
-                    }
-                    mma_commit(mbar);
+        for (int ci = 0; ci < 2; ci++) {
+            if (pair < npair && el < nelt) {
+                const float* q = xin + (el * CIN + ci) * NP + 8 * (j + 8 * k) + i0;
+                if (vec) {
+                    const float4 u = __ldg(reinterpret_cast<const float4*>(q));
+                    x[ci][0] = u.x, x[ci][1] = u.y, x[ci][2] = u.z, x[ci][3] = u.w;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; i++) x[ci][i] = __ldg(q + i);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; i++) x[ci][i] = 0.f;
+            }
+        }
+    };
+    int64_t pair = blockIdx.x + (int64_t)gridDim.x * grp;
+    load_line(pair);
+    for (; pair < npair; pair += step) {
+        const int64_t el = 2 * pair + e;
+        const bool live = el < nelt;
+        // input: channels 0, 1 of the line's rows (rounded to BF16), channels 2..15 zero
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const __nv_bfloat162 x01 = __floats2bfloat162_rn(x[0][i], x[1][i]);
+            *reinterpret_cast<uint4*>(rows + i * kPoint) =
+                make_uint4(*reinterpret_cast<const uint32_t*>(&x01), 0u, 0u, 0u);
+            *reinterpret_cast<uint4*>(rows + i * kPoint + kHalf) = make_uint4(0, 0, 0, 0);
+        }
+        bool failed = false;  // uniform across the group (decided by its barrier)
+        for (int layer = 0; layer < 3; layer++) {
+            tc5::fence_async_smem();  // the rows, written by this group's threads, are read by the tensor core
+            tc5::fence_before();
+            group_sync(grp);
+            tc5::fence_after();
+            if ((warp & 7) == 0) {
+                if (tc5::elect_one()) {
+                    layer_mmas(d_tile, a0, b0 + (uint64_t)(layer * (9 * kTap >> 4)));
+                    tc5::mma_commit(mbar);
                 }
                 __syncwarp();
             }
-            bool ok = mbar_wait_bounded(mbar, parity, wait_ns);
-            if (__syncthreads_or(!ok)) {
-                // a wait ran out: flag it, poison the element's output, wait once more for the MMAs in
-                // flight, then leave the element loop (TMEM is freed below)
-                failed = true;
-                if (tid == 0) {
-                    atomicExch(&g_net_tc5_timeout, 1);
-                    z[e * NP] = __longlong_as_double(0x7FF8000000000000LL);
+            double2 cv[2];
+            double sc = 0.0;
+            if (layer == 2) {  // under the last layer's MMAs: the next pair's input, this pair's output factors
+                load_line(pair + step);
+                if (live) {
+                    sc = (double)scale[el];
+                    const double* cl = c + el * NP + 8 * (j + 8 * k) + i0;
+#pragma unroll
+                    for (int i = 0; i < 4; i += 2)
+                        cv[i / 2] = vecz ? __ldg(reinterpret_cast<const double2*>(cl + i))
+                                         : make_double2(__ldg(cl + i), __ldg(cl + i + 1));
                 }
-                mbar_wait_bounded(mbar, parity, wait_ns);
+            }
+            // the group's first warp waits for the MMAs, the others for it at the barrier
+            const bool ok = (warp & 7) != 0 || tc5::mbar_wait_bounded(mbar, parity, wait_ns, kHint);
+            if (group_or(grp, !ok)) {
+                // a wait ran out: flag it, poison the pair's outputs, wait once more for the MMAs in
+                // flight, then leave the loop (TMEM is freed below)
+                failed = true;
+                if (m == 0) atomicExch(&g_net_tc5_timeout, 1);
+                if (j == 0 && k == 0 && i0 == 0 && live) z[el * NP] = __longlong_as_double(0x7FF8000000000000LL);
+                tc5::mbar_wait_bounded(mbar, parity, wait_ns);
                 break;
             }
             parity ^= 1u;
-            tc_fence_after();
+            __syncwarp();
+            tc5::fence_after();
+            if (layer < 2) {
+                const float* b = layer == 0 ? S.b1 : S.b2;
 #pragma unroll 1
-            for (int tile = 0; tile < kTiles; tile++) {
-                float v[16];
-                tmem_ld16(lane_addr + 16u * (uint32_t)tile, v);
-                const int lout = 16 * tile + (m >> 3), i = m & 7, jp = lout % 10, k = lout / 10;
-                if (jp < 1 || jp > 8) continue;  // a padding line of the output: dropped
-                if (layer < 2) {
-                    const float* b = layer == 0 ? S.b1 : S.b2;
+                for (int i = 0; i < 4; i++) {
+                    float v[16];
+                    tc5::tmem_ld16(lane_addr + 16u * (uint32_t)i, v);
                     uint32_t packed[8];
 #pragma unroll
                     for (int q = 0; q < 8; q++) {
@@ -272,25 +280,34 @@ __global__ void __launch_bounds__(NT5, 3) k_net_apply_tc5(int64_t nelt, const fl
                             __floats2bfloat162_rn(gelu5(v[2 * q] + b[2 * q]), gelu5(v[2 * q + 1] + b[2 * q + 1]));
                         packed[q] = *reinterpret_cast<const uint32_t*>(&h2);
                     }
-                    const int off = grid_row(i + 1, jp, k + 1);
-                    *reinterpret_cast<uint4*>(act + off) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                    *reinterpret_cast<uint4*>(act + kHalfBytes + off) =
+                    *reinterpret_cast<uint4*>(rows + i * kPoint) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+                    *reinterpret_cast<uint4*>(rows + i * kPoint + kHalf) =
                         make_uint4(packed[4], packed[5], packed[6], packed[7]);
-                } else {
-                    const int p = i + 8 * (jp - 1) + 64 * k;
-                    z[e * NP + p] = (double)(v[0] + S.b3[0]) * sc * c[e * NP + p];
+                }
+            } else {
+                float y[4];
+                tmem_ld_points(lane_addr, y);
+                if (live) {
+                    double* zl = z + el * NP + 8 * (j + 8 * k) + i0;
+#pragma unroll
+                    for (int i = 0; i < 4; i += 2) {
+                        const double2 v = make_double2((double)(y[i] + S.b3[0]) * sc * cv[i / 2].x,
+                                                       (double)(y[i + 1] + S.b3[0]) * sc * cv[i / 2].y);
+                        if (vecz)
+                            *reinterpret_cast<double2*>(zl + i) = v;
+                        else
+                            zl[i] = v.x, zl[i + 1] = v.y;
+                    }
                 }
             }
-            tc_fence_before();
+            tc5::fence_before();
         }
         if (failed) break;
-        __syncthreads();  // the next element's input overwrites the grid
     }
-    tc_fence_before();
+    tc5::fence_before();
     __syncthreads();
-    tc_fence_after();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    tc5::fence_after();
+    if (warp == 0) tc5::tmem_dealloc(tmem, kTmemCols);
 }
 
 int sm_count()
@@ -315,9 +332,10 @@ nek_status launch_net_apply_tc5_ex(int64_t nelt, const float* theta, const float
     static std::atomic<uint64_t> configured{0};
     nek_status st = ensure_dyn_smem(k_net_apply_tc5, sizeof(Tc5Smem), configured);
     if (st != NEK_OK) return st;
-    const int64_t cap = 3 * (int64_t)sm_count();
-    const int grid = static_cast<int>(nelt < cap ? nelt : cap);
-    k_net_apply_tc5<<<grid, NT5, sizeof(Tc5Smem), s>>>(nelt, theta, xin, scale, c, z, wait_ns, arrivals);
+    const int64_t npair = (nelt + 1) / 2, cap = sm_count();  // one CTA per SM, a pair for every SM before a second group's
+    const int grid = static_cast<int>(npair < cap ? npair : cap);
+    k_net_apply_tc5<<<grid, kGroups * kGroupThreads, sizeof(Tc5Smem), s>>>(nelt, theta, xin, scale, c, z, wait_ns,
+                                                                          arrivals);
     return check_launch();
 }
 

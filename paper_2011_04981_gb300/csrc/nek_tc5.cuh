@@ -72,6 +72,14 @@ __device__ __forceinline__ void mma_commit_lane0(uint32_t mbar)
         : "memory");
 }
 
+// True in one thread of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+    return r != 0;
+}
+
 // The mbarrier gets one arrival once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint32_t mbar)
 {

@@ -394,3 +394,26 @@ def test_trained_network_beats_untrained_and_jacobi():
     assert lrn["iters"] < unt["iters"], (lrn, unt)
     assert lrn["iters"] < jac["iters"], (lrn, jac)
     assert lrn["fell_back_at"] == 0
+
+
+@pytest.mark.parametrize("n,shift", [(1, 0), (2, 0), (3, 1), (305, 0), (913, 0), (914, 1)])
+def test_apply_bf16_pairs_and_groups(n, shift):
+    """Elements go through the tensor cores two at a time, three pairs per SM: an element's output is that of a call with
+    this element alone, to the bit, whatever its place, a last pair of one element and inputs that are not 16-byte
+    aligned (shift: elements of the arrays' types) included; nothing is written past the end."""
+    rng = np.random.default_rng(n)
+    th = torch.from_numpy(_theta(3).astype(np.float32)).to(DEV)
+    xin = torch.from_numpy(rng.normal(size=n * 1024 + shift).astype(np.float32)).to(DEV)[shift:]
+    sc = torch.from_numpy(rng.uniform(0.1, 2.0, size=n).astype(np.float32)).to(DEV)
+    c = torch.from_numpy(rng.uniform(0.1, 1.0, size=n * 512 + shift)).to(DEV)[shift:]
+    z = torch.full((n * 512 + shift + 8,), -7.0, dtype=torch.float64, device=DEV)
+    nekax.net_apply_bf16(n, 8, th, xin, sc, c, z[shift:])
+    torch.cuda.synchronize()
+    assert torch.all(z[shift + n * 512:] == -7.0) and torch.all(z[:shift] == -7.0)
+    z = z[shift:shift + n * 512]
+    assert torch.all(torch.isfinite(z))
+    one = torch.empty(512, dtype=torch.float64, device=DEV)
+    for e in sorted({0, 1, 2, n // 3, n // 2, n - 2, n - 1} & set(range(n))):
+        nekax.net_apply_bf16(1, 8, th, xin[e * 1024:].contiguous(), sc[e:].contiguous(), c[e * 512:].contiguous(), one)
+        torch.cuda.synchronize()
+        assert torch.equal(one, z[e * 512:(e + 1) * 512]), e
