@@ -44,29 +44,6 @@ __device__ __forceinline__ void stage_weights(const float* __restrict__ W, float
     }
 }
 
-// acc[o] = bias[o] + sum_c sum_t W[o][c][t] x[c][p + t] for point p = (i, j, k).
-template <int CI, int CO>
-__device__ __forceinline__ void conv_point(const float* xin, const float* sW, const float* sb, int i, int j, int k,
-                                           float (&acc)[CO])
-{
-#pragma unroll
-    for (int o = 0; o < CO; o++) acc[o] = sb[o];
-#pragma unroll
-    for (int t = 0; t < 27; t++) {
-        const int dk = t / 9 - 1, dj = (t / 3) % 3 - 1, di = t % 3 - 1;
-        const int ii = i + di, jj = j + dj, kk = k + dk;
-        if (ii < 0 || ii >= NXN || jj < 0 || jj >= NXN || kk < 0 || kk >= NXN) continue;
-        const int q = ii + NXN * (jj + NXN * kk);
-#pragma unroll 4
-        for (int c = 0; c < CI; c++) {
-            const float xv = xin[c * NP + q];
-            const float* w = sW + (c * 27 + t) * CO;
-#pragma unroll
-            for (int o = 0; o < CO; o++) acc[o] = fmaf(w[o], xv, acc[o]);
-        }
-    }
-}
-
 // Two points per thread, p and p + NP/2 (planes k and k + 4): every weight read
 // from shared memory feeds two FMAs.
 template <int CI, int CO>
@@ -214,51 +191,237 @@ __global__ void __launch_bounds__(NT_APPLY) k_net_apply(int64_t nelt, const floa
 }
 
 // ------------------------------------------------------------------ training
-// Forward over a batch of B samples keeping the pre-activations h1, h2 and y.
-__global__ void __launch_bounds__(NP) k_net_fwd_train(int B, const float* __restrict__ theta,
-                                                      const float* __restrict__ xin, float* __restrict__ h1,
-                                                      float* __restrict__ h2, float* __restrict__ y)
+//
+// The convolutions and their gradients work on lines of 8 points along i.  A thread holds a line of one input
+// channel in registers and feeds 22 multiply-adds (three taps along i, the zero padding at its ends left out) from it
+// for each of four output channels: 88 multiply-adds for five 16-byte shared-memory loads (convolution), or 22 for each of
+// 16 channel pairs from 16 loads (weight gradient).  A block is one sample and a quarter of the output channels, 256
+// threads, so that a batch of 256 spreads evenly (1024 blocks over 152 SMs) and a small one still fills the chip; the
+// 16 input channels are shared out over four groups of 64 threads, whose sums are added through shared memory.
+//
+// What bounds it: the FP32 pipe (12 M multiply-adds a sample and their recomputed part, 80 us a batch of 256 at the
+// pipe's rate).  A batch of 256: forward 62 + 10 us, backward 15 + 96 us, a whole energy-norm gradient 209 us; one block of 512
+// threads a sample, one point or one 4 x 4 tile of channel pairs a thread, took 91, 536 and 654 us.
+constexpr int NTT = 256;    // threads of the training kernels: 64 lines x 4 groups
+constexpr int CS = 520;     // floats of one channel in shared memory: 64 lines and a zero line
+constexpr int kZeroLine = 512;
+
+// The two 16-byte halves of a line are exchanged in lines j = 4..7, so that eight lanes on consecutive lines meet all banks:
+// place of the first half (float index; the second is at ^ 4).
+__device__ __forceinline__ int line_at(int j, int k) { return 8 * (j + 8 * k) + ((j & 4) ? 4 : 0); }
+// The nine neighbours (dj, dk) of line (j, k); the zero line outside the element.
+__device__ __forceinline__ void line_neighbours(int j, int k, int (&off)[9])
+{
+#pragma unroll
+    for (int q = 0; q < 9; q++) {
+        const int jj = j + q % 3 - 1, kk = k + q / 3 - 1;
+        off[q] = jj >= 0 && jj < 8 && kk >= 0 && kk < 8 ? line_at(jj, kk) : kZeroLine;
+    }
+}
+__device__ __forceinline__ void line_load(const float* s, int at, float (&x)[8])
+{
+    const float4 a = *reinterpret_cast<const float4*>(s + at), b = *reinterpret_cast<const float4*>(s + (at ^ 4));
+    x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w;
+    x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
+}
+__device__ __forceinline__ void line_store(float* s, int at, const float (&x)[8])
+{
+    *reinterpret_cast<float4*>(s + at) = make_float4(x[0], x[1], x[2], x[3]);
+    *reinterpret_cast<float4*>(s + (at ^ 4)) = make_float4(x[4], x[5], x[6], x[7]);
+}
+__device__ __forceinline__ void line_load_global(const float* g, float (&x)[8])
+{
+#pragma unroll
+    for (int i = 0; i < 8; i++) x[i] = g[i];
+}
+
+// The same for the workspace's arrays, which are 16-byte aligned.
+__device__ __forceinline__ void line_load_ws(const float* g, float (&x)[8])
+{
+    const float4 a = *reinterpret_cast<const float4*>(g), b = *reinterpret_cast<const float4*>(g + 4);
+    x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w;
+    x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
+}
+__device__ __forceinline__ void line_store_ws(float* g, const float (&x)[8])
+{
+    *reinterpret_cast<float4*>(g) = make_float4(x[0], x[1], x[2], x[3]);
+    *reinterpret_cast<float4*>(g + 4) = make_float4(x[4], x[5], x[6], x[7]);
+}
+
+// acc[o][p] += sum over the CN channels from s on and the 27 taps of w x: four output channels of one line.  sW:
+// [channel][dj, dk][di][4 outputs].
+template <int CN>
+__device__ __forceinline__ void conv4(const float* s, const float* sW, const int (&off)[9], float (&acc)[4][8])
+{
+#pragma unroll 1
+    for (int c = 0; c < CN; c++) {
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+            float x[8];
+            line_load(s + c * CS, off[q], x);
+            const float4* wq = reinterpret_cast<const float4*>(sW) + (c * 9 + q) * 3;
+            const float4 wm = wq[0], w0 = wq[1], wp = wq[2];
+            const float m[4] = {wm.x, wm.y, wm.z, wm.w}, z[4] = {w0.x, w0.y, w0.z, w0.w}, n[4] = {wp.x, wp.y, wp.z, wp.w};
+#pragma unroll
+            for (int o = 0; o < 4; o++)
+#pragma unroll
+                for (int p = 0; p < 8; p++) {
+                    if (p > 0) acc[o][p] = fmaf(m[o], x[p - 1], acc[o][p]);
+                    acc[o][p] = fmaf(z[o], x[p], acc[o][p]);
+                    if (p < 7) acc[o][p] = fmaf(n[o], x[p + 1], acc[o][p]);
+                }
+        }
+    }
+}
+
+// acc[di] += sum_p g[p] x[p + di] over one line.
+__device__ __forceinline__ void corr3(const float (&g)[8], const float (&x)[8], float (&acc)[3])
+{
+#pragma unroll
+    for (int p = 0; p < 8; p++) {
+        if (p > 0) acc[0] = fmaf(g[p], x[p - 1], acc[0]);
+        acc[1] = fmaf(g[p], x[p], acc[1]);
+        if (p < 7) acc[2] = fmaf(g[p], x[p + 1], acc[2]);
+    }
+}
+
+// Sums the four groups' acc of output channel `grp` through red (4 x 4 x 512 floats); every thread gets its line of it.
+__device__ __forceinline__ void group_sum(float* red, int grp, int at, const float (&acc)[4][8], float (&out)[8])
+{
+    __syncthreads();
+#pragma unroll
+    for (int o = 0; o < 4; o++) line_store(red + (grp * 4 + o) * 512, at, acc[o]);
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < 8; p++) out[p] = 0.f;
+#pragma unroll
+    for (int g = 0; g < 4; g++) {
+        float x[8];
+        line_load(red + (g * 4 + grp) * 512, at, x);
+#pragma unroll
+        for (int p = 0; p < 8; p++) out[p] += x[p];
+    }
+}
+
+// Weights of four outputs o0 .. o0 + 3 over CI channels as [channel][dj, dk][di][4]; FLIP: the taps of the transposed
+// convolution, with W's roles exchanged (W[channel][o] read at the mirrored tap).
+template <int CI, bool FLIP>
+__device__ __forceinline__ void stage_conv4(const float* __restrict__ W, int o0, int nin, float* sW)
+{
+    for (int q = threadIdx.x; q < CI * 27 * 4; q += NTT) {
+        const int o = o0 + (q & 3), t = (q >> 2) % 27, c = q / 108;
+        sW[q] = bf16r(FLIP ? W[(c * nin + o) * 27 + 26 - t] : W[(o * nin + c) * 27 + t]);
+    }
+}
+
+struct Fwd12Smem {
+    float a1[CH * CS];  // later the group sums
+    float x[CIN * CS];
+    float w1[4 * CIN * 108];
+    float w2[CH * 108];
+    float b1[CH], b2[4];
+};
+
+// Layers 1 and 2 of sample blockIdx.x / 4; writes channels 4 q .. 4 q + 3 (q = blockIdx.x % 4) of the pre-activations h1, h2.
+__global__ void __launch_bounds__(NTT, 3) k_net_fwd12(const float* __restrict__ theta, const float* __restrict__ xin,
+                                                      float* __restrict__ h1, float* __restrict__ h2)
 {
     extern __shared__ __align__(16) unsigned char raw[];
-    ApplySmem& S = *reinterpret_cast<ApplySmem*>(raw);
-    stage_weights<CIN, CH>(theta + OW1, S.w1);
-    stage_weights<CH, CH>(theta + OW2, S.w2);
-    stage_weights<CH, 1>(theta + OW3, S.w3);
-    if (threadIdx.x < CH) {
-        S.b1[threadIdx.x] = bf16r(theta[OB1 + threadIdx.x]);
-        S.b2[threadIdx.x] = bf16r(theta[OB2 + threadIdx.x]);
+    Fwd12Smem& S = *reinterpret_cast<Fwd12Smem*>(raw);
+    const int64_t b = blockIdx.x >> 2;
+    const int part = blockIdx.x & 3, tid = threadIdx.x, grp = tid >> 6, l = tid & 63, j = l & 7, k = l >> 3;
+    for (int g = 0; g < 4; g++) stage_conv4<CIN, false>(theta + OW1, 4 * g, CIN, S.w1 + g * CIN * 108);
+    stage_conv4<CH, false>(theta + OW2, 4 * part, CH, S.w2);
+    if (tid < CH) S.b1[tid] = bf16r(theta[OB1 + tid]);
+    if (tid < 4) S.b2[tid] = bf16r(theta[OB2 + 4 * part + tid]);
+    const int at = line_at(j, k);
+    if (grp < CIN) {
+        float v[8];
+        line_load_global(xin + (b * CIN + grp) * NP + 8 * l, v);
+        line_store(S.x + grp * CS, at, v);
     }
-    if (threadIdx.x == 0) S.b3[0] = bf16r(theta[OB3]);
-    const int p = threadIdx.x;
-    const int i = p % NXN, j = (p / NXN) % NXN, k = p / (NXN * NXN);
-    for (int b = blockIdx.x; b < B; b += gridDim.x) {
-        __syncthreads();
-        S.x[p] = xin[(b * CIN + 0) * NP + p];
-        S.x[NP + p] = xin[(b * CIN + 1) * NP + p];
-        __syncthreads();
-        {
-            float acc[CH];
-            conv_point<CIN, CH>(S.x, S.w1, S.b1, i, j, k, acc);
+    if (tid < CIN * 8) S.x[(tid >> 3) * CS + kZeroLine + (tid & 7)] = 0.f;
+    if (tid < CH * 8) S.a1[(tid >> 3) * CS + kZeroLine + (tid & 7)] = 0.f;
+    int off[9];
+    line_neighbours(j, k, off);
+    __syncthreads();
+    float acc[4][8];
 #pragma unroll
-            for (int o = 0; o < CH; o++) {
-                h1[((int64_t)b * CH + o) * NP + p] = acc[o];
-                S.a1[o * NP + p] = gelu(acc[o]);
+    for (int o = 0; o < 4; o++)
+#pragma unroll
+        for (int p = 0; p < 8; p++) acc[o][p] = S.b1[4 * grp + o];
+    conv4<CIN>(S.x, S.w1 + grp * CIN * 108, off, acc);
+#pragma unroll
+    for (int o = 0; o < 4; o++) {
+        if (grp == part) line_store_ws(h1 + (b * CH + 4 * grp + o) * NP + 8 * l, acc[o]);
+#pragma unroll
+        for (int p = 0; p < 8; p++) acc[o][p] = gelu(acc[o][p]);
+        line_store(S.a1 + (4 * grp + o) * CS, at, acc[o]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int o = 0; o < 4; o++)
+#pragma unroll
+        for (int p = 0; p < 8; p++) acc[o][p] = 0.f;
+    conv4<4>(S.a1 + 4 * grp * CS, S.w2 + 4 * grp * 108, off, acc);
+    float out[8];
+    group_sum(S.a1, grp, at, acc, out);
+    const float bias = S.b2[grp];
+#pragma unroll
+    for (int p = 0; p < 8; p++) out[p] += bias;
+    line_store_ws(h2 + (b * CH + 4 * part + grp) * NP + 8 * l, out);
+}
+
+struct Fwd3Smem {
+    float a2[CH * CS];
+    float red[4 * 512];
+    float w3[CH * 28];  // [channel][tap], padded
+    float b3[4];
+};
+
+// Layer 3 of sample blockIdx.x: y from the pre-activations h2.
+__global__ void __launch_bounds__(NTT) k_net_fwd3(const float* __restrict__ theta, const float* __restrict__ h2,
+                                                  float* __restrict__ y)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    Fwd3Smem& S = *reinterpret_cast<Fwd3Smem*>(raw);
+    const int64_t b = blockIdx.x;
+    const int tid = threadIdx.x, grp = tid >> 6, l = tid & 63, j = l & 7, k = l >> 3, at = line_at(j, k);
+    for (int q = tid; q < CH * 27; q += NTT) S.w3[q / 27 * 28 + q % 27] = bf16r(theta[OW3 + q]);
+    if (tid == 0) S.b3[0] = bf16r(theta[OB3]);
+    if (tid < CH * 8) S.a2[(tid >> 3) * CS + kZeroLine + (tid & 7)] = 0.f;
+#pragma unroll
+    for (int a = 0; a < 4; a++) {
+        float v[8];
+        line_load_ws(h2 + (b * CH + 4 * grp + a) * NP + 8 * l, v);
+#pragma unroll
+        for (int p = 0; p < 8; p++) v[p] = gelu(v[p]);
+        line_store(S.a2 + (4 * grp + a) * CS, at, v);
+    }
+    int off[9];
+    line_neighbours(j, k, off);
+    __syncthreads();
+    float acc[8] = {};
+#pragma unroll 1
+    for (int c = 4 * grp; c < 4 * grp + 4; c++) {
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+            float x[8];
+            line_load(S.a2 + c * CS, off[q], x);
+            const float* w = S.w3 + c * 28 + 3 * q;
+#pragma unroll
+            for (int p = 0; p < 8; p++) {
+                if (p > 0) acc[p] = fmaf(w[0], x[p - 1], acc[p]);
+                acc[p] = fmaf(w[1], x[p], acc[p]);
+                if (p < 7) acc[p] = fmaf(w[2], x[p + 1], acc[p]);
             }
         }
-        __syncthreads();
-        {
-            float acc[CH];
-            conv_point<CH, CH>(S.a1, S.w2, S.b2, i, j, k, acc);
-#pragma unroll
-            for (int o = 0; o < CH; o++) {
-                h2[((int64_t)b * CH + o) * NP + p] = acc[o];
-                S.a2[o * NP + p] = gelu(acc[o]);
-            }
-        }
-        __syncthreads();
-        float yo[1];
-        conv_point<CH, 1>(S.a2, S.w3, S.b3, i, j, k, yo);
-        y[(int64_t)b * NP + p] = yo[0];
+    }
+    line_store(S.red + grp * 512, at, acc);
+    __syncthreads();
+    for (int q = tid; q < NP; q += NTT) {
+        const int i = q & 7, jj = (q >> 3) & 7, a = line_at(jj, q >> 6), r = (i < 4 ? a : a ^ 4) + (i & 3);
+        y[b * NP + q] = ((S.red[r] + S.red[512 + r]) + (S.red[1024 + r] + S.red[1536 + r])) + S.b3[0];
     }
 }
 
@@ -333,182 +496,282 @@ __global__ void __launch_bounds__(NP) k_net_energy_loss(int B, const float* __re
     }
 }
 
-struct BwdSmem {
-    float x[CIN * NP];
-    float a1[CH * NP];
-    float g2[CH * NP];  // a2, then dh2
-    float g1[CH * NP];  // dh1
-    float dy[NP];
-    float w2[CH * 27 * CH];  // [c][t][o]
-    float w3[CH * 27];       // [c][t]
+// Weight-gradient tasks: (dj, dk) x channel tile x line group, 9 x 4 x 7 of the 256 threads.  A tile holds the
+// channels ct, ct + 4, ct + 8, ct + 12, which lie on different banks.
+constexpr int kLineGroups = 7;
+
+struct Bwd3Smem {
+    float a2[CH * CS];
+    float dy[CS];
+    float w3[4 * 108];
+    float red[36 * 12 * kLineGroups];
+    float sum[NTT / 32];
 };
 
-// d/dx of sum_p g[o][p] * conv(x)[o][p] at input channel c, point q:
-// sum_o sum_t W[o][c][t] g[o][q - t]  (W staged as [c][t][o])
-template <int CO>
-__device__ __forceinline__ float convT_point(const float* g, const float* sW, int c, int i, int j, int k)
+// Backward of layer 3 of sample blockIdx.x: dW3, db3 into gs, and h2 (the pre-activations) replaced by
+// dh2 = gelu'(h2) convT(dy; W3).
+__global__ void __launch_bounds__(NTT, 2) k_net_bwd3(const float* __restrict__ theta, const float* __restrict__ dy,
+                                                     float* __restrict__ h2, float* __restrict__ gs)
 {
-    float s = 0.f;
-#pragma unroll
-    for (int t = 0; t < 27; t++) {
-        const int dk = t / 9 - 1, dj = (t / 3) % 3 - 1, di = t % 3 - 1;
-        const int ii = i - di, jj = j - dj, kk = k - dk;
-        if (ii < 0 || ii >= NXN || jj < 0 || jj >= NXN || kk < 0 || kk >= NXN) continue;
-        const int q = ii + NXN * (jj + NXN * kk);
-        const float* w = sW + (c * 27 + t) * CO;
-#pragma unroll
-        for (int o = 0; o < CO; o++) s = fmaf(w[o], g[o * NP + q], s);
+    extern __shared__ __align__(16) unsigned char raw[];
+    Bwd3Smem& S = *reinterpret_cast<Bwd3Smem*>(raw);
+    const int64_t b = blockIdx.x;
+    float* g = gs + b * NPARAM;
+    const int tid = threadIdx.x, grp = tid >> 6, l = tid & 63, j = l & 7, k = l >> 3, at = line_at(j, k);
+    // [group][dj, dk][di][4 channels] of the mirrored taps
+    for (int q = tid; q < 4 * 108; q += NTT) {
+        const int c = 4 * (q / 108) + (q & 3), t = (q % 108) >> 2;
+        S.w3[q] = bf16r(theta[OW3 + c * 27 + 26 - t]);
     }
-    return s;
-}
-
-// dW[o][c][t] = sum_p g[o][p] x[c][p + t] for a 4x4 (o, c) tile and one tap per thread.
-template <int CI>
-__device__ __forceinline__ void wgrad_tiles(const float* g, const float* x, int CO, float* out /*[CO][CI][27]*/)
-{
-    const int otiles = (CO + 3) / 4, ctiles = (CI + 3) / 4;
-    const int ntask = otiles * ctiles * 27;
-    for (int task = threadIdx.x; task < ntask; task += blockDim.x) {
-        const int t = task % 27, ct = (task / 27) % ctiles, ot = task / (27 * ctiles);
-        const int dk = t / 9 - 1, dj = (t / 3) % 3 - 1, di = t % 3 - 1;
-        float acc[4][4] = {};
-        for (int p = 0; p < NP; p++) {
-            const int i = p % NXN, j = (p / NXN) % NXN, k = p / (NXN * NXN);
-            const int ii = i + di, jj = j + dj, kk = k + dk;
-            if (ii < 0 || ii >= NXN || jj < 0 || jj >= NXN || kk < 0 || kk >= NXN) continue;
-            const int q = ii + NXN * (jj + NXN * kk);
-            float gv[4], xv[4];
+    float sdy = 0.f;
+    if (grp == 0) {
+        float v[8];
+        line_load_ws(dy + b * NP + 8 * l, v);
+        line_store(S.dy, at, v);
+#pragma unroll
+        for (int p = 0; p < 8; p++) sdy += v[p];
+    }
+    if (tid < 8) S.dy[kZeroLine + tid] = 0.f;
+    if (tid < CH * 8) S.a2[(tid >> 3) * CS + kZeroLine + (tid & 7)] = 0.f;
+    float gp[4][8];
+#pragma unroll
+    for (int a = 0; a < 4; a++) {
+        float v[8];
+        line_load_ws(h2 + (b * CH + 4 * grp + a) * NP + 8 * l, v);
+#pragma unroll
+        for (int p = 0; p < 8; p++) {
+            gp[a][p] = gelu_grad(v[p]);
+            v[p] = gelu(v[p]);
+        }
+        line_store(S.a2 + (4 * grp + a) * CS, at, v);
+    }
+    if (grp == 0) {  // db3: two warps
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sdy += __shfl_xor_sync(0xffffffffu, sdy, o);
+        if ((tid & 31) == 0) S.sum[tid >> 5] = sdy;
+    }
+    int off[9];
+    line_neighbours(j, k, off);
+    __syncthreads();
+    if (tid == 0) g[OB3] = S.sum[0] + S.sum[1];
+    {
+        float acc[4][8] = {};
+        conv4<1>(S.dy, S.w3 + grp * 108, off, acc);
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+#pragma unroll
+            for (int p = 0; p < 8; p++) acc[a][p] *= gp[a][p];
+            line_store_ws(h2 + (b * CH + 4 * grp + a) * NP + 8 * l, acc[a]);
+        }
+    }
+    // dW3[c][t] = sum_p dy a2(p + t)
+    if (tid < 36 * kLineGroups) {
+        const int ct = tid & 3, q = (tid >> 2) % 9, lg = tid / 36, dj = q % 3 - 1, dk = q / 3 - 1;
+        float acc[4][3] = {};
+#pragma unroll 1
+        for (int m = lg; m < 64; m += kLineGroups) {
+            const int jj = (m & 7) + dj, kk = (m >> 3) + dk;
+            const int xo = jj >= 0 && jj < 8 && kk >= 0 && kk < 8 ? line_at(jj, kk) : kZeroLine;
+            float gv[8];
+            line_load(S.dy, line_at(m & 7, m >> 3), gv);
 #pragma unroll
             for (int a = 0; a < 4; a++) {
-                const int o = ot * 4 + a, c = ct * 4 + a;
-                gv[a] = o < CO ? g[o * NP + p] : 0.f;
-                xv[a] = c < CI ? x[c * NP + q] : 0.f;
+                float x[8];
+                line_load(S.a2 + (ct + 4 * a) * CS, xo, x);
+                corr3(gv, x, acc[a]);
             }
-#pragma unroll
-            for (int a = 0; a < 4; a++)
-#pragma unroll
-                for (int bb = 0; bb < 4; bb++) acc[a][bb] = fmaf(gv[a], xv[bb], acc[a][bb]);
         }
 #pragma unroll
         for (int a = 0; a < 4; a++)
 #pragma unroll
-            for (int bb = 0; bb < 4; bb++) {
-                const int o = ot * 4 + a, c = ct * 4 + bb;
-                if (o < CO && c < CI) out[(o * CI + c) * 27 + t] = acc[a][bb];
-            }
+            for (int d = 0; d < 3; d++) S.red[lg * 432 + (ct + 4 * a) * 27 + 3 * q + d] = acc[a][d];
+    }
+    __syncthreads();
+    for (int q = tid; q < CH * 27; q += NTT) {
+        float v = 0.f;
+#pragma unroll
+        for (int lg = 0; lg < kLineGroups; lg++) v += S.red[lg * 432 + q];
+        g[OW3 + q] = v;
     }
 }
 
-// Backward for one sample per block iteration: per-sample gradient vector gs[b][NPARAM].
-__global__ void __launch_bounds__(NP) k_net_bwd(int B, const float* __restrict__ theta,
-                                                const float* __restrict__ xin, const float* __restrict__ h1,
-                                                const float* __restrict__ h2, const float* __restrict__ dy,
-                                                float* __restrict__ gs)
+struct Bwd12Smem {
+    float g2[CH * CS];  // dh2
+    float a1[CH * CS];  // gelu(h1); later the partial sums
+    float x[CIN * CS];
+    float g1[4 * CS];   // dh1, this quarter's channels
+    float w2[CH * 108];
+};
+static_assert(36 * 24 * kLineGroups <= CH * CS && 16 * 512 <= CH * CS && 9 * 24 * 28 <= CH * CS, "partial sums fit");
+
+// Backward of layers 2 and 1 of sample blockIdx.x / 4 for a quarter q = blockIdx.x % 4 of the channels: dW2 and db2 of the
+// outputs 4 q .. 4 q + 3, and dh1 = gelu'(h1) convT(dh2; W2), dW1 and db1 of the hidden channels 4 q .. 4 q + 3.
+__global__ void __launch_bounds__(NTT, 2)
+    k_net_bwd12(const float* __restrict__ theta, const float* __restrict__ xin, const float* __restrict__ h1,
+                const float* __restrict__ dh2, float* __restrict__ gs)
 {
     extern __shared__ __align__(16) unsigned char raw[];
-    BwdSmem& S = *reinterpret_cast<BwdSmem*>(raw);
-    stage_weights<CH, CH>(theta + OW2, S.w2);
-    stage_weights<CH, 1>(theta + OW3, S.w3);
-    const int p = threadIdx.x;
-    const int i = p % NXN, j = (p / NXN) % NXN, k = p / (NXN * NXN);
-    __shared__ float red[CH][NP / 32];
-    for (int b = blockIdx.x; b < B; b += gridDim.x) {
-        float* g = gs + (int64_t)b * NPARAM;
-        __syncthreads();
-        S.x[p] = xin[(b * CIN + 0) * NP + p];
-        S.x[NP + p] = xin[(b * CIN + 1) * NP + p];
-        S.dy[p] = dy[(int64_t)b * NP + p];
+    Bwd12Smem& S = *reinterpret_cast<Bwd12Smem*>(raw);
+    const int64_t b = blockIdx.x >> 2;
+    float* g = gs + b * NPARAM;
+    const int part = blockIdx.x & 3, tid = threadIdx.x, grp = tid >> 6, l = tid & 63, j = l & 7, k = l >> 3;
+    const int at = line_at(j, k);
+    stage_conv4<CH, true>(theta + OW2, 4 * part, CH, S.w2);
+    if (grp < CIN) {
+        float v[8];
+        line_load_global(xin + (b * CIN + grp) * NP + 8 * l, v);
+        line_store(S.x + grp * CS, at, v);
+    }
+    if (tid < CIN * 8) S.x[(tid >> 3) * CS + kZeroLine + (tid & 7)] = 0.f;
+    if (tid < CH * 8) {
+        S.g2[(tid >> 3) * CS + kZeroLine + (tid & 7)] = 0.f;
+        S.a1[(tid >> 3) * CS + kZeroLine + (tid & 7)] = 0.f;
+    }
+#pragma unroll 2
+    for (int a = 0; a < 4; a++) {
+        float v[8];
+        line_load_ws(dh2 + (b * CH + 4 * grp + a) * NP + 8 * l, v);
+        line_store(S.g2 + (4 * grp + a) * CS, at, v);
+        line_load_ws(h1 + (b * CH + 4 * grp + a) * NP + 8 * l, v);
 #pragma unroll
-        for (int o = 0; o < CH; o++) {
-            S.a1[o * NP + p] = gelu(h1[((int64_t)b * CH + o) * NP + p]);
-            S.g2[o * NP + p] = gelu(h2[((int64_t)b * CH + o) * NP + p]);
-        }
-        __syncthreads();
-        // layer 3: dW3 = sum_p dy a2(p + t); db3 = sum dy
-        wgrad_tiles<CH>(S.dy, S.g2, 1, g + OW3);
-        __syncthreads();
-        // dh2 = gelu'(h2) * convT(dy; W3)
+        for (int p = 0; p < 8; p++) v[p] = gelu(v[p]);
+        line_store(S.a1 + (4 * grp + a) * CS, at, v);
+    }
+    __syncthreads();
+    // ---- dW2[o][c][t] = sum_p dh2[o] a1[c](p + t): four outputs x a tile of four channels x three taps a thread
+    const int ct = tid & 3, q9 = (tid >> 2) % 9, lg = tid / 36, dj = q9 % 3 - 1, dk = q9 / 3 - 1;
+    {
+        float acc[4][4][3] = {};
+        if (tid < 36 * kLineGroups) {
+#pragma unroll 1
+            for (int m = lg; m < 64; m += kLineGroups) {
+                const int jj = (m & 7) + dj, kk = (m >> 3) + dk;
+                const int xo = jj >= 0 && jj < 8 && kk >= 0 && kk < 8 ? line_at(jj, kk) : kZeroLine;
+                const int go = line_at(m & 7, m >> 3);
+                float gv[4][8];
 #pragma unroll
-        for (int c = 0; c < CH; c++) {
-            const float v = convT_point<1>(S.dy, S.w3, c, i, j, k);
-            S.g2[c * NP + p] = v * gelu_grad(h2[((int64_t)b * CH + c) * NP + p]);
-        }
-        __syncthreads();
-        // layer 2: dW2 = sum_p dh2 a1(p + t)
-        wgrad_tiles<CH>(S.g2, S.a1, CH, g + OW2);
-        // dh1 = gelu'(h1) * convT(dh2; W2)
-#pragma unroll 4
-        for (int c = 0; c < CH; c++) {
-            const float v = convT_point<CH>(S.g2, S.w2, c, i, j, k);
-            S.g1[c * NP + p] = v * gelu_grad(h1[((int64_t)b * CH + c) * NP + p]);
-        }
-        __syncthreads();
-        // layer 1: dW1 = sum_p dh1 x(p + t)
-        wgrad_tiles<CIN>(S.g1, S.x, CH, g + OW1);
-        // biases: sums over the block's points (fixed shuffle tree)
-        {
-            float v3 = S.dy[p];
-            float v2[CH], v1[CH];
+                for (int o = 0; o < 4; o++) line_load(S.g2 + (4 * part + o) * CS, go, gv[o]);
 #pragma unroll
-            for (int o = 0; o < CH; o++) {
-                v2[o] = S.g2[o * NP + p];
-                v1[o] = S.g1[o * NP + p];
-            }
+                for (int a = 0; a < 4; a++) {
+                    float x[8];
+                    line_load(S.a1 + (ct + 4 * a) * CS, xo, x);
 #pragma unroll
-            for (int s = 16; s > 0; s >>= 1) {
-                v3 += __shfl_xor_sync(0xffffffffu, v3, s);
-#pragma unroll
-                for (int o = 0; o < CH; o++) {
-                    v2[o] += __shfl_xor_sync(0xffffffffu, v2[o], s);
-                    v1[o] += __shfl_xor_sync(0xffffffffu, v1[o], s);
+                    for (int o = 0; o < 4; o++) corr3(gv[o], x, acc[o][a]);
                 }
             }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; h++) {  // two outputs at a time through the space of a1
             __syncthreads();
-            if ((p & 31) == 0) {
-                red[0][p >> 5] = v3;
+            if (tid < 36 * kLineGroups) {
+#pragma unroll
+                for (int o = 0; o < 2; o++)
+#pragma unroll
+                    for (int a = 0; a < 4; a++)
+#pragma unroll
+                        for (int d = 0; d < 3; d++)
+                            S.a1[lg * 864 + (o * CH + ct + 4 * a) * 27 + 3 * q9 + d] = acc[2 * h + o][a][d];
             }
             __syncthreads();
-            if (p == 0) {
-                float s = 0.f;
-                for (int q = 0; q < NP / 32; q++) s += red[0][q];
-                g[OB3] = s;
-            }
-            __syncthreads();
-            if ((p & 31) == 0)
-                for (int o = 0; o < CH; o++) red[o][p >> 5] = v2[o];
-            __syncthreads();
-            if (p < CH) {
-                float s = 0.f;
-                for (int q = 0; q < NP / 32; q++) s += red[p][q];
-                g[OB2 + p] = s;
-            }
-            __syncthreads();
-            if ((p & 31) == 0)
-                for (int o = 0; o < CH; o++) red[o][p >> 5] = v1[o];
-            __syncthreads();
-            if (p < CH) {
-                float s = 0.f;
-                for (int q = 0; q < NP / 32; q++) s += red[p][q];
-                g[OB1 + p] = s;
+            for (int q = tid; q < 864; q += NTT) {
+                float v = 0.f;
+#pragma unroll
+                for (int n = 0; n < kLineGroups; n++) v += S.a1[n * 864 + q];
+                g[OW2 + (4 * part + 2 * h) * CH * 27 + q] = v;
             }
         }
+    }
+    // ---- dh1 of this quarter
+    {
+        int off[9];
+        line_neighbours(j, k, off);
+        float acc[4][8] = {};
+        conv4<4>(S.g2 + 4 * grp * CS, S.w2 + 4 * grp * 108, off, acc);
+        float out[8], hv[8];
+        group_sum(S.a1, grp, at, acc, out);
+        line_load_ws(h1 + (b * CH + 4 * part + grp) * NP + 8 * l, hv);
+#pragma unroll
+        for (int p = 0; p < 8; p++) out[p] *= gelu_grad(hv[p]);
+        line_store(S.g1 + grp * CS, at, out);
+    }
+    __syncthreads();
+    // ---- biases: a warp for each of the quarter's channels of dh2 and dh1
+    {
+        const int w = tid >> 5, lane = tid & 31;
+        const float* src = w < 4 ? S.g2 + (4 * part + w) * CS : S.g1 + (w - 4) * CS;
+        float v = 0.f;
+#pragma unroll
+        for (int q = 0; q < NP / 32; q++) v += src[lane + 32 * q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) g[w < 4 ? OB2 + 4 * part + w : OB1 + 4 * part + w - 4] = v;
+    }
+    // ---- dW1[o][c][t] = sum_p dh1[o] x[c](p + t): all 24 of a (dj, dk) a thread, 28 line groups
+    if (tid < 9 * 28) {
+        const int q = tid % 9, n = tid / 9, d1 = q % 3 - 1, d2 = q / 3 - 1;
+        float acc[4][CIN][3] = {};
+#pragma unroll 1
+        for (int m = n; m < 64; m += 28) {
+            const int jj = (m & 7) + d1, kk = (m >> 3) + d2;
+            const int xo = jj >= 0 && jj < 8 && kk >= 0 && kk < 8 ? line_at(jj, kk) : kZeroLine;
+            const int go = line_at(m & 7, m >> 3);
+            float x[CIN][8];
+#pragma unroll
+            for (int c = 0; c < CIN; c++) line_load(S.x + c * CS, xo, x[c]);
+#pragma unroll
+            for (int o = 0; o < 4; o++) {
+                float gv[8];
+                line_load(S.g1 + o * CS, go, gv);
+#pragma unroll
+                for (int c = 0; c < CIN; c++) corr3(gv, x[c], acc[o][c]);
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < 4; o++)
+#pragma unroll
+            for (int c = 0; c < CIN; c++)
+#pragma unroll
+                for (int d = 0; d < 3; d++) S.a1[n * 216 + (o * CIN + c) * 27 + 3 * q + d] = acc[o][c][d];
+    }
+    __syncthreads();
+    for (int q = tid; q < 4 * CIN * 27; q += NTT) {
+        float v = 0.f;
+#pragma unroll
+        for (int n = 0; n < 28; n++) v += S.a1[n * 216 + q];
+        g[OW1 + 4 * part * CIN * 27 + q] = v;
     }
 }
 
-// grad[q] = sum_b gs[b][q] in order; loss = sum_b loss_b / B.
-__global__ void k_net_reduce(int B, const float* __restrict__ gs, const float* __restrict__ loss_b,
-                             float* __restrict__ grad, float* __restrict__ loss)
+// grad[q] = sum_b gs[b][q], loss = sum_b loss_b / B: 32 parameters a block, the samples shared out over eight warps
+// (warp w takes b = w, w + 8, ...), whose sums are added in order.  The loads' latency is what a thread waits
+// for: 256 samples one after the other took 17 us.
+constexpr int kReduceWarps = 8;
+__global__ void __launch_bounds__(32 * kReduceWarps) k_net_reduce(int B, const float* __restrict__ gs,
+                                                                  const float* __restrict__ loss_b,
+                                                                  float* __restrict__ grad, float* __restrict__ loss)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ float sh[2][kReduceWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
+    const bool with_loss = blockIdx.x == 0 && loss;
+    float s = 0.f, sl = 0.f;
     if (q < NPARAM) {
-        float s = 0.f;
-        for (int b = 0; b < B; b++) s += gs[(int64_t)b * NPARAM + q];
-        grad[q] = s;
+#pragma unroll 16
+        for (int b = w; b < B; b += kReduceWarps) s += gs[(int64_t)b * NPARAM + q];
     }
-    if (q == 0 && loss) {
-        float s = 0.f;
-        for (int b = 0; b < B; b++) s += loss_b[b];
-        loss[0] = s / (float)B;
+    if (with_loss && lane == 0) {
+#pragma unroll 16
+        for (int b = w; b < B; b += kReduceWarps) sl += loss_b[b];
+    }
+    sh[0][w][lane] = s;
+    sh[1][w][lane] = sl;
+    __syncthreads();
+    if (w == 0) {
+        for (int k = 1; k < kReduceWarps; k++) {
+            s += sh[0][k][lane];
+            sl += sh[1][k][lane];
+        }
+        if (q < NPARAM) grad[q] = s;
+        if (with_loss && lane == 0) loss[0] = sl / (float)B;
     }
 }
 
@@ -525,9 +788,35 @@ __global__ void k_adam(int n, float* __restrict__ th, const float* __restrict__ 
     th[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + eps);
 }
 
-std::atomic<uint64_t> g_apply_conf{0}, g_fwd_conf{0}, g_bwd_conf{0};
+std::atomic<uint64_t> g_apply_conf{0}, g_fwd12_conf{0}, g_fwd3_conf{0}, g_bwd3_conf{0}, g_bwd12_conf{0};
 
 int grid_for(int64_t n) { return static_cast<int>(n < 152 * 2 ? n : 152 * 2); }
+
+// Forward pass of a batch, keeping the pre-activations.
+nek_status launch_train_forward(int batch, const float* theta, const float* xin, float* h1, float* h2, float* y,
+                                cudaStream_t s)
+{
+    nek_status st = ensure_dyn_smem(k_net_fwd12, sizeof(Fwd12Smem), g_fwd12_conf);
+    if (st == NEK_OK) st = ensure_dyn_smem(k_net_fwd3, sizeof(Fwd3Smem), g_fwd3_conf);
+    if (st != NEK_OK) return st;
+    k_net_fwd12<<<4u * (unsigned)batch, NTT, sizeof(Fwd12Smem), s>>>(theta, xin, h1, h2);
+    k_net_fwd3<<<(unsigned)batch, NTT, sizeof(Fwd3Smem), s>>>(theta, h2, y);
+    return check_launch();
+}
+
+// Backward pass from dy: each sample's gradient into gs; h2 is overwritten.  Then the sums over the batch.
+nek_status launch_train_backward(int batch, const float* theta, const float* xin, const float* h1, float* h2,
+                                 const float* dy, float* gs, const float* lossb, float* grad, float* loss,
+                                 cudaStream_t s)
+{
+    nek_status st = ensure_dyn_smem(k_net_bwd3, sizeof(Bwd3Smem), g_bwd3_conf);
+    if (st == NEK_OK) st = ensure_dyn_smem(k_net_bwd12, sizeof(Bwd12Smem), g_bwd12_conf);
+    if (st != NEK_OK) return st;
+    k_net_bwd3<<<(unsigned)batch, NTT, sizeof(Bwd3Smem), s>>>(theta, dy, h2, gs);
+    k_net_bwd12<<<4u * (unsigned)batch, NTT, sizeof(Bwd12Smem), s>>>(theta, xin, h1, h2, gs);
+    k_net_reduce<<<(NPARAM + 31) / 32, 32 * kReduceWarps, 0, s>>>(batch, gs, lossb, grad, loss);
+    return check_launch();
+}
 
 }  // namespace
 
@@ -641,10 +930,7 @@ nek_status nek_net_forward_batch(int batch, const float* theta, const float* xin
     if (batch <= 0 || !theta || !xin || !y || !workspace || !is_aligned(workspace, 256)) return NEK_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     TrainLayout L = train_layout(static_cast<char*>(workspace), batch);
-    nek_status st = ensure_dyn_smem(k_net_fwd_train, sizeof(ApplySmem), g_fwd_conf);
-    if (st != NEK_OK) return st;
-    k_net_fwd_train<<<grid_for(batch), NP, sizeof(ApplySmem), s>>>(batch, theta, xin, L.h1, L.h2, y);
-    return check_launch();
+    return launch_train_forward(batch, theta, xin, L.h1, L.h2, y, s);
 }
 
 nek_status nek_net_train_grad(int batch, const float* theta, const float* xin, const float* target, float* grad,
@@ -654,14 +940,10 @@ nek_status nek_net_train_grad(int batch, const float* theta, const float* xin, c
         return NEK_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     TrainLayout L = train_layout(static_cast<char*>(workspace), batch);
-    nek_status st0 = ensure_dyn_smem(k_net_fwd_train, sizeof(ApplySmem), g_fwd_conf);
-    if (st0 == NEK_OK) st0 = ensure_dyn_smem(k_net_bwd, sizeof(BwdSmem), g_bwd_conf);
-    if (st0 != NEK_OK) return st0;
-    k_net_fwd_train<<<grid_for(batch), NP, sizeof(ApplySmem), s>>>(batch, theta, xin, L.h1, L.h2, L.y);
+    const nek_status st = launch_train_forward(batch, theta, xin, L.h1, L.h2, L.y, s);
+    if (st != NEK_OK) return st;
     k_net_loss<<<grid_for(batch), NP, 0, s>>>(batch, L.y, target, L.dy, L.lossb);
-    k_net_bwd<<<grid_for(batch), NP, sizeof(BwdSmem), s>>>(batch, theta, xin, L.h1, L.h2, L.dy, L.gs);
-    k_net_reduce<<<(NPARAM + 255) / 256, 256, 0, s>>>(batch, L.gs, L.lossb, grad, loss);
-    return check_launch();
+    return launch_train_backward(batch, theta, xin, L.h1, L.h2, L.dy, L.gs, L.lossb, grad, loss, s);
 }
 
 nek_status nek_net_train_grad_energy(int batch, const float* theta, const float* xin, const float* target,
@@ -673,20 +955,15 @@ nek_status nek_net_train_grad_energy(int batch, const float* theta, const float*
         return NEK_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     TrainLayout L = train_layout(static_cast<char*>(workspace), batch);
-    nek_status st0 = ensure_dyn_smem(k_net_fwd_train, sizeof(ApplySmem), g_fwd_conf);
-    if (st0 == NEK_OK) st0 = ensure_dyn_smem(k_net_bwd, sizeof(BwdSmem), g_bwd_conf);
-    if (st0 != NEK_OK) return st0;
     const int64_t n = (int64_t)batch * NP;
-    k_net_fwd_train<<<grid_for(batch), NP, sizeof(ApplySmem), s>>>(batch, theta, xin, L.h1, L.h2, L.y);
-    k_net_diff<<<pcg::stream_blocks(n), 256, 0, s>>>(n, L.y, target, L.d);
-    nek_status st = check_launch();
+    nek_status st = launch_train_forward(batch, theta, xin, L.h1, L.h2, L.y, s);
     if (st != NEK_OK) return st;
+    k_net_diff<<<pcg::stream_blocks(n), 256, 0, s>>>(n, L.y, target, L.d);
+    if ((st = check_launch()) != NEK_OK) return st;
     if ((st = launch_ax_lowp(NEK_PREC_F32, batch, NXN, D, Glp32, gscale, L.d, L.Ad, s)) != NEK_OK) return st;
     if ((st = launch_ax_lowp(NEK_PREC_F32, batch, NXN, D, Glp32, gscale, target, L.At, s)) != NEK_OK) return st;
     k_net_energy_loss<<<grid_for(batch), NP, 0, s>>>(batch, L.d, L.Ad, target, L.At, L.dy, L.lossb);
-    k_net_bwd<<<grid_for(batch), NP, sizeof(BwdSmem), s>>>(batch, theta, xin, L.h1, L.h2, L.dy, L.gs);
-    k_net_reduce<<<(NPARAM + 255) / 256, 256, 0, s>>>(batch, L.gs, L.lossb, grad, loss);
-    return check_launch();
+    return launch_train_backward(batch, theta, xin, L.h1, L.h2, L.dy, L.gs, L.lossb, grad, loss, s);
 }
 
 nek_status nek_adam_step(int n, float* theta, const float* grad, float* m, float* v, float lr, float beta1,

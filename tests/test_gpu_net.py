@@ -417,3 +417,35 @@ def test_apply_bf16_pairs_and_groups(n, shift):
         nekax.net_apply_bf16(1, 8, th, xin[e * 1024:].contiguous(), sc[e:].contiguous(), c[e * 512:].contiguous(), one)
         torch.cuda.synchronize()
         assert torch.equal(one, z[e * 512:(e + 1) * 512]), e
+
+
+@pytest.mark.parametrize("B,shift,with_loss", [(1, 0, True), (3, 1, False), (9, 0, True), (41, 3, True)])
+def test_gradient_batch_sizes_and_alignment(B, shift, with_loss):
+    """Batches of one sample, fewer and more than the eight warps that sum them; inputs at any 4-byte address; loss left
+    out: every gradient entry inside the oracle's bounds."""
+    rng = np.random.default_rng(50 + B)
+    th = _theta(6)
+    x = rng.normal(size=(B, 2, 8, 8, 8)).astype(np.float32)
+    t = rng.normal(size=(B, 8, 8, 8)).astype(np.float32)
+    xd = torch.zeros(x.size + shift, dtype=torch.float32, device=DEV)
+    td = torch.zeros(t.size + shift, dtype=torch.float32, device=DEV)
+    xd[shift:] = torch.from_numpy(x.reshape(-1)).to(DEV)
+    td[shift:] = torch.from_numpy(t.reshape(-1)).to(DEV)
+    ws = torch.empty(nekax.net_train_workspace_bytes(B) // 4 + 64, dtype=torch.float32, device=DEV)
+    g = torch.full((onet.NPARAM,), float("nan"), dtype=torch.float32, device=DEV)
+    loss = torch.full((1,), -1.0, dtype=torch.float32, device=DEV)
+    nekax.net_train_grad(B, torch.from_numpy(th.astype(np.float32)).to(DEV), xd[shift:], td[shift:], g,
+                         loss if with_loss else None, ws)
+    torch.cuda.synchronize()
+    L, gr, worst = onet.loss_and_grad_bound(th, x.astype(np.float64), t.astype(np.float64), mode="worst")
+    _, _, rms = onet.loss_and_grad_bound(th, x.astype(np.float64), t.astype(np.float64), mode="rms")
+    if with_loss:
+        assert abs(float(loss.item()) - L) <= 1e-4 * L
+    else:
+        assert float(loss.item()) == -1.0
+    gg = g.cpu().numpy().astype(np.float64)
+    o = 0
+    for name, shp in onet.SHAPES:
+        n = int(np.prod(shp))
+        _check_elementwise("grad " + name, gg[o:o + n], gr[o:o + n], worst[o:o + n], rms[o:o + n])
+        o += n
