@@ -318,30 +318,6 @@ __global__ void __launch_bounds__(BT) kb_p(const int64_t* __restrict__ ch_begin,
     }
 }
 
-__global__ void k_bdiag_local(int64_t nelt, int nx, const double* __restrict__ D, const double* __restrict__ G,
-                              double* __restrict__ d)
-{
-    const int64_t n3 = (int64_t)nx * nx * nx;
-    for (int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; gid < nelt * n3;
-         gid += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = gid / n3;
-        const int p = static_cast<int>(gid - e * n3);
-        const int i = p % nx, j = (p / nx) % nx, k = p / (nx * nx);
-        const double* Ge = G + e * n3 * 6;
-        double s = 0.0;
-        for (int l = 0; l < nx; l++) {
-            const double a = D[l * nx + i], b = D[l * nx + j], cc = D[l * nx + k];
-            s += Ge[6 * (l + nx * (j + nx * k)) + 0] * a * a;
-            s += Ge[6 * (i + nx * (l + nx * k)) + 3] * b * b;
-            s += Ge[6 * (i + nx * (j + nx * l)) + 5] * cc * cc;
-        }
-        const double* g = Ge + 6 * p;
-        const double di = D[i * nx + i], dj = D[j * nx + j], dk = D[k * nx + k];
-        s += 2.0 * (g[1] * di * dj + g[2] * di * dk + g[4] * dj * dk);
-        d[gid] = s;
-    }
-}
-
 __global__ void k_binvert(int64_t n, const uint8_t* __restrict__ mask, double* __restrict__ d)
 {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
@@ -595,14 +571,9 @@ nek_status nek_batch_jacobi_minv(const nek_batch* b, const double* G, const uint
 {
     if (!b || !G || !mask || !minv || !is_aligned(G, 16) || !is_aligned(minv, 8)) return NEK_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    for (const auto& g : b->groups) {
-        const int64_t n = g.nelt * (int64_t)g.nx * g.nx * g.nx;
-        const int64_t nb = (n + 255) / 256;
-        k_bdiag_local<<<static_cast<int>(std::min<int64_t>(nb, 152 * 16)), 256, 0, s>>>(
-            g.nelt, g.nx, g.D, G + g.pt0 * 6, minv + g.pt0);
-    }
-    nek_status st = check_launch();
-    if (st != NEK_OK) return st;
+    nek_status st = NEK_OK;
+    for (const auto& g : b->groups)
+        if ((st = launch_diag_local(g.nelt, g.nx, g.D, G + g.pt0 * 6, minv + g.pt0, s)) != NEK_OK) return st;
     if ((st = pcg::dssum<double>(b->gs, minv, s)) != NEK_OK) return st;
     k_binvert<<<pcg::stream_blocks(b->npts), 256, 0, s>>>(b->npts, mask, minv);
     return check_launch();
