@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_dot_c_partials(int64_t n, co
                                                                    const double* __restrict__ b,
                                                                    double* __restrict__ parts)
 {
-    __shared__ double sh[kReduceThreads / 32];
+    __shared__ double sh[kReduceThreads];
     double acc = 0.0;
     for (int64_t p = blockIdx.x * (int64_t)kReduceThreads + threadIdx.x; p < n;
          p += (int64_t)gridDim.x * kReduceThreads)
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_dot_c_partials(int64_t n, co
 __global__ void __launch_bounds__(kReduceThreads) k_sum_partials(const double* __restrict__ parts, int nparts,
                                                                  double* __restrict__ out)
 {
-    __shared__ double sh[kReduceThreads / 32];
+    __shared__ double sh[kReduceThreads];
     double t = sum_partials<kReduceThreads>(parts, nparts, sh);
     if (threadIdx.x == 0) out[0] = t;
 }

@@ -52,32 +52,13 @@ struct Group {
 
 __device__ __forceinline__ bool bhalted(const BScal& s) { return s.done || s.status != NEK_OK; }
 
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 template <int NA>
 __device__ __forceinline__ void chunk_reduce(double (&acc)[NA], double* parts, int nchunks, int cid)
 {
-    __shared__ double sh[NA][BT / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int a = 0; a < NA; a++) {
-        const double v = warp_sum(acc[a]);
-        if (lane == 0) sh[a][wid] = v;
-    }
-    __syncthreads();
-    if (wid == 0) {
-#pragma unroll
-        for (int a = 0; a < NA; a++) {
-            double t = lane < BT / 32 ? sh[a][lane] : 0.0;
-            t = warp_sum(t);
-            if (lane == 0) parts[a * nchunks + cid] = t;
-        }
-    }
+    __shared__ double sh[NA * BT];
+    const double t = block_sums<BT, NA>(acc, sh);
+    const int a = threadIdx.x >> 5;
+    if (a < NA && (threadIdx.x & 31) == 0) parts[a * nchunks + cid] = t;
 }
 
 // x = 0; r = mask.f; p = z = minv r; partials <r,z>, <r,r>
@@ -112,25 +93,41 @@ __device__ __forceinline__ int chunk_of(const int32_t* __restrict__ clist)
     return clist ? clist[blockIdx.x] : static_cast<int>(blockIdx.x);
 }
 
-// one warp per problem: sums its partials [c0, c1) in order
+// One block per problem sums its partials [c0, c1) of both halves of parts (or of parts alone) in a fixed order; valid in
+// thread 0.
+constexpr int PT = 128;
 template <class I>
 __device__ __forceinline__ double prob_sum(const double* __restrict__ parts, I c0, I c1)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ double sh[PT];
     double v = 0.0;
 #pragma unroll 4
-    for (I q = c0 + lane; q < c1; q += 32) v += parts[q];
-    return warp_sum(v);
+    for (I q = c0 + static_cast<int>(threadIdx.x); q < c1; q += PT) v += parts[q];
+    return block_sum<PT>(v, sh);
+}
+__device__ __forceinline__ void prob_sum2(const double* __restrict__ parts, int nchunks, int c0, int c1, double& a,
+                                          double& b)
+{
+    __shared__ double sh[2 * PT];
+    double v[2] = {0.0, 0.0};
+    for (int q = c0 + static_cast<int>(threadIdx.x); q < c1; q += PT) {
+        v[0] += parts[q];
+        v[1] += parts[nchunks + q];
+    }
+    const double t = block_sums<PT, 2>(v, sh);
+    if (threadIdx.x == 32) sh[0] = t;
+    __syncthreads();
+    a = t;
+    b = sh[0];
 }
 
-__global__ void kb_init_finish(int nprob, const int* __restrict__ pch, const double* __restrict__ parts, int nchunks,
-                               double tol, BScal* __restrict__ sc, int* __restrict__ active)
+__global__ void __launch_bounds__(PT) kb_init_finish(const int* __restrict__ pch, const double* __restrict__ parts,
+                                                     int nchunks, double tol, BScal* __restrict__ sc, int* __restrict__ active)
 {
-    const int pid = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    if (pid >= nprob) return;
-    const double rz = prob_sum(parts, pch[pid], pch[pid + 1]);
-    const double rr = prob_sum(parts + nchunks, pch[pid], pch[pid + 1]);
-    if ((threadIdx.x & 31) == 0) {
+    const int pid = blockIdx.x;
+    double rz, rr;
+    prob_sum2(parts, nchunks, pch[pid], pch[pid + 1], rz, rr);
+    if (threadIdx.x == 0) {
         BScal s{};
         s.rz = rz;
         s.rr = rr;
@@ -170,18 +167,17 @@ __global__ void __launch_bounds__(BT) kb_pw(const int64_t* __restrict__ ch_begin
 
 // pw from the chunk partials of kb_pw or, with edot, from the element energies
 // of the float-float operator (problem p's elements are [pel[p], pel[p+1]))
-__global__ void kb_alpha(int nprob, const int* __restrict__ pch, const double* __restrict__ parts,
-                         BScal* __restrict__ sc, int* __restrict__ active, const int64_t* __restrict__ pel,
+__global__ void __launch_bounds__(PT) kb_alpha(const int* __restrict__ pch, const double* __restrict__ parts,
+                                               BScal* __restrict__ sc, int* __restrict__ active, const int64_t* __restrict__ pel,
                          const double* __restrict__ edot)
 {
-    const int pid = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    if (pid >= nprob) return;
+    const int pid = blockIdx.x;
     if (bhalted(sc[pid])) {
-        if ((threadIdx.x & 31) == 0) sc[pid].xpend = 0;
+        if (threadIdx.x == 0) sc[pid].xpend = 0;
         return;
     }
     const double pw = edot ? prob_sum(edot, pel[pid], pel[pid + 1]) : prob_sum(parts, pch[pid], pch[pid + 1]);
-    if ((threadIdx.x & 31) == 0) {
+    if (threadIdx.x == 0) {
         BScal& s = sc[pid];
         s.it += 1;
         s.pw = pw;
@@ -231,14 +227,14 @@ __global__ void __launch_bounds__(BT) kb_update(const int64_t* __restrict__ ch_b
     chunk_reduce<2>(acc, parts, nchunks, c);
 }
 
-__global__ void kb_beta(int nprob, const int* __restrict__ pch, const double* __restrict__ parts, int nchunks,
-                        BScal* __restrict__ sc, int* __restrict__ active)
+__global__ void __launch_bounds__(PT) kb_beta(const int* __restrict__ pch, const double* __restrict__ parts, int nchunks,
+                                              BScal* __restrict__ sc, int* __restrict__ active)
 {
-    const int pid = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    if (pid >= nprob || bhalted(sc[pid])) return;
-    const double rr = prob_sum(parts, pch[pid], pch[pid + 1]);
-    const double rz = prob_sum(parts + nchunks, pch[pid], pch[pid + 1]);
-    if ((threadIdx.x & 31) == 0) {
+    const int pid = blockIdx.x;
+    if (bhalted(sc[pid])) return;
+    double rr, rz;
+    prob_sum2(parts, nchunks, pch[pid], pch[pid + 1], rr, rz);
+    if (threadIdx.x == 0) {
         BScal& s = sc[pid];
         s.rr = rr;
         s.relres = sqrt(rr) / s.bnorm;
@@ -597,7 +593,6 @@ nek_status nek_batch_cg_solve(const nek_batch* b, const double* G, const float* 
     nek_status st = NEK_OK;
     const double* mv = minv;
     const int nc = b->nchunks, np = b->nprob;
-    const int wblocks = (np + 7) / 8;  // 8 warps (problems) per 256-thread block
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     int it_done = 0, launches = 0, graph_launches = 0;
@@ -640,9 +635,9 @@ nek_status nek_batch_cg_solve(const nek_batch* b, const double* G, const float* 
                                             b->gs->d_members, L.w, gl);
         // the float-float operator writes element energies, which give <p,w> (no kb_pw pass)
         if (!Gff) kb_pw<<<n_act, BT, 0, ss>>>(b->d_ch_begin, b->d_ch_prob, nc, L.flags, L.p, L.w, L.parts, L.sc, cl);
-        kb_alpha<<<wblocks, 256, 0, ss>>>(np, b->d_pch, L.parts, L.sc, L.active, b->d_pel, Gff ? L.edot : nullptr);
+        kb_alpha<<<np, PT, 0, ss>>>(b->d_pch, L.parts, L.sc, L.active, b->d_pel, Gff ? L.edot : nullptr);
         kb_update<<<n_act, BT, 0, ss>>>(b->d_ch_begin, b->d_ch_prob, nc, L.flags, mv, L.w, L.r, L.parts, L.sc, cl);
-        kb_beta<<<wblocks, 256, 0, ss>>>(np, b->d_pch, L.parts, nc, L.sc, L.active);
+        kb_beta<<<np, PT, 0, ss>>>(b->d_pch, L.parts, nc, L.sc, L.active);
         kb_test<<<(np + 255) / 256, 256, 0, ss>>>(np, tol_rel, L.sc, L.active, L.pdone);
         kb_p<<<n_act, BT, 0, ss>>>(b->d_ch_begin, b->d_ch_prob, mv, L.r, x, L.p, L.sc, cl);
         iter_launches += (n_gact > 0 ? 1 : 0) + (Gff ? 0 : 1) + 5;
@@ -735,7 +730,7 @@ nek_status nek_batch_cg_solve(const nek_batch* b, const double* G, const float* 
     if ((st = pcg::build_flags(b->gs, b->npts, mask, L.flags, s)) != NEK_OK) goto done;
     launches += b->gs->ngroups > 0 ? 2 : 1;
     kb_init<<<nc, BT, 0, s>>>(b->d_ch_begin, b->d_ch_prob, nc, L.flags, mv, f, x, L.r, L.p, L.parts);
-    kb_init_finish<<<wblocks, 256, 0, s>>>(np, b->d_pch, L.parts, nc, tol_rel, L.sc, L.active);
+    kb_init_finish<<<np, PT, 0, s>>>(b->d_pch, L.parts, nc, tol_rel, L.sc, L.active);
     kb_test<<<(np + 255) / 256, 256, 0, s>>>(np, tol_rel, L.sc, L.active, L.pdone);  // initial pdone
     launches += 3;
     if ((st = check_launch()) != NEK_OK) goto done;

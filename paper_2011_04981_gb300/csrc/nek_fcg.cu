@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(NT) kf_init(int64_t n, const double* __restric
                                               double* __restrict__ x, double* __restrict__ r,
                                               double* __restrict__ parts)
 {
-    __shared__ double sh[NT / 32];
+    __shared__ double sh[2 * NT];
     double acc = 0.0;
     for (int64_t q = blockIdx.x * (int64_t)NT + threadIdx.x; q < n; q += (int64_t)gridDim.x * NT) {
         const double rq = mask[q] ? f[q] : 0.0;
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(NT) kf_init(int64_t n, const double* __restric
 
 __global__ void __launch_bounds__(NT) kf_rr(const double* __restrict__ parts, int nb, int first, FScal* sc)
 {
-    __shared__ double sh[NT / 32];
+    __shared__ double sh[2 * NT];
     const double rr = sum_partials<NT>(parts, nb, sh);
     if (threadIdx.x == 0) {
         sc->rr = rr;
@@ -93,7 +93,8 @@ __global__ void __launch_bounds__(NT) kf_zdots(int64_t n, const double* __restri
                                                const double* __restrict__ Wbase, int64_t stride, Window win,
                                                double* __restrict__ parts)
 {
-    __shared__ double sh[NT / 32];
+    constexpr int R = M < NT / 32 ? (M > 0 ? M : 1) : NT / 32;  // sums reduced together, a warp each
+    __shared__ double sh[R * NT];
     const double* W[M > 0 ? M : 1];
 #pragma unroll
     for (int i = 0; i < M; i++) W[i] = Wbase + win.slot[i] * stride;
@@ -115,20 +116,23 @@ __global__ void __launch_bounds__(NT) kf_zdots(int64_t n, const double* __restri
         for (int i = 0; i < M; i++) acc[i] += cz * wv[i];
     }
 #pragma unroll
-    for (int i = 0; i < M; i++) {
-        const double t = block_sum<NT>(acc[i], sh);
-        if (threadIdx.x == 0) parts[i * gridDim.x + blockIdx.x] = t;
+    for (int i = 0; i < M; i += R) {
+        double v[R];
+#pragma unroll
+        for (int k = 0; k < R; k++) v[k] = i + k < M ? acc[i + k < M ? i + k : 0] : 0.0;
+        const double t = block_sums<NT, R>(v, sh);
+        const int k = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0 && k < R && i + k < M) parts[(i + k) * gridDim.x + blockIdx.x] = t;
     }
 }
 
 // beta_i = <z, W_i> / <p_i, W_i>
 __global__ void __launch_bounds__(NT) kf_betas(const double* __restrict__ parts, int nb, Window win, FScal* sc)
 {
-    __shared__ double sh[NT / 32];
-    for (int i = 0; i < win.n; i++) {
-        const double d = sum_partials<NT>(parts + i * nb, nb, sh);
-        if (threadIdx.x == 0) sc->beta[i] = d / sc->pwv[win.slot[i]];
-    }
+    __shared__ double sh[NT];
+    const int i = blockIdx.x;  // one block for each of the window's directions
+    const double d = sum_partials<NT>(parts + i * nb, nb, sh);
+    if (threadIdx.x == 0) sc->beta[i] = d / sc->pwv[win.slot[i]];
 }
 
 // P_cur = z - sum_i beta_i P_i (the window's M directions)
@@ -166,7 +170,7 @@ nek_status window_kernels(int64_t n, int nb, int sb, const double* c, const uint
             return window_kernels<M + 1>(n, nb, sb, c, mask, z, P, W, stride, cur, win, parts, sc, s, launches);
     }
     kf_zdots<M><<<nb, NT, 0, s>>>(n, c, mask, z, W, stride, win, parts);
-    if (M > 0) kf_betas<<<1, NT, 0, s>>>(parts, nb, win, sc);
+    if (M > 0) kf_betas<<<M, NT, 0, s>>>(parts, nb, win, sc);
     kf_p<M><<<sb, 256, 0, s>>>(n, z, P, stride, cur, win, sc);
     *launches += M > 0 ? 3 : 2;
     return check_launch();
@@ -177,7 +181,7 @@ __global__ void __launch_bounds__(NT) kf_pw(int64_t n, const double* __restrict_
                                             const double* __restrict__ p, double* __restrict__ w,
                                             const double* __restrict__ r, double* __restrict__ parts)
 {
-    __shared__ double sh[NT / 32];
+    __shared__ double sh[2 * NT];
     double a = 0.0, b = 0.0;
     for (int64_t q = blockIdx.x * (int64_t)NT + threadIdx.x; q < n; q += (int64_t)gridDim.x * NT) {
         double wq = w[q];
@@ -189,17 +193,14 @@ __global__ void __launch_bounds__(NT) kf_pw(int64_t n, const double* __restrict_
         a += cp * wq;
         b += cp * r[q];
     }
-    double t = block_sum<NT>(a, sh);
-    if (threadIdx.x == 0) parts[blockIdx.x] = t;
-    t = block_sum<NT>(b, sh);
-    if (threadIdx.x == 0) parts[gridDim.x + blockIdx.x] = t;
+    write_two_partials<NT>(a, b, parts, sh);
 }
 
 __global__ void __launch_bounds__(NT) kf_alpha(const double* __restrict__ parts, int nb, int cur, FScal* sc)
 {
-    __shared__ double sh[NT / 32];
-    const double pw = sum_partials<NT>(parts, nb, sh);
-    const double pr = sum_partials<NT>(parts + nb, nb, sh);
+    __shared__ double sh[2 * NT];
+    double pw, pr;
+    sum_two_partials<NT>(parts, nb, sh, pw, pr);
     if (threadIdx.x == 0) {
         sc->pw = pw;
         sc->pr = pr;
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(NT) kf_update(int64_t n, const double* __restr
                                                 double* __restrict__ x, double* __restrict__ r,
                                                 double* __restrict__ parts, const FScal* __restrict__ sc)
 {
-    __shared__ double sh[NT / 32];
+    __shared__ double sh[2 * NT];
     const double alpha = sc->alpha;
     double acc = 0.0;
     for (int64_t q = blockIdx.x * (int64_t)NT + threadIdx.x; q < n; q += (int64_t)gridDim.x * NT) {

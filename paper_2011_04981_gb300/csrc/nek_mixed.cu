@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(NT) k_mix_init(int64_t n, const double* __rest
                                                   double* __restrict__ x, double* __restrict__ r,
                                                   double* __restrict__ parts)
 {
-    __shared__ double sh[NT / 32];
+    __shared__ double sh[NT];
     double acc = 0.0;
     for (int64_t q = blockIdx.x * (int64_t)NT + threadIdx.x; q < n; q += (int64_t)gridDim.x * NT) {
         const double rq = mask[q] ? f[q] : 0.0;
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(NT) k_mix_residual(int64_t n, const double* __
                                                       const double* __restrict__ w, double* __restrict__ r,
                                                       double* __restrict__ parts)
 {
-    __shared__ double sh[NT / 32];
+    __shared__ double sh[NT];
     double acc = 0.0;
     for (int64_t q = blockIdx.x * (int64_t)NT + threadIdx.x; q < n; q += (int64_t)gridDim.x * NT) {
         const double rq = mask[q] ? f[q] - w[q] : 0.0;
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(NT) k_mix_residual(int64_t n, const double* __
 __global__ void __launch_bounds__(NT) k_mix_norm(const double* __restrict__ parts, int nb, int first,
                                                   MixScalars* ms)
 {
-    __shared__ double sh[NT / 32];
+    __shared__ double sh[NT];
     const double rr = sum_partials<NT>(parts, nb, sh);
     if (threadIdx.x == 0) {
         ms->rnorm = sqrt(rr);
