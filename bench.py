@@ -43,6 +43,9 @@ sys.path.insert(0, ROOT)
 METRIC = "AX GDOF/s & % HBM peak; CG s-to-1e-8 residual, FP64 vs mixed/learned"
 UNIT = "GDOF/s"
 FP64_PEAK_TFLOPS = 1.2586  # 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz (nominal 1.25 TFLOP/s)
+# FP64 instructions a point of nek_ax from nx = 3 on (the product with G 9, the sum of three directions 2); its
+# contractions run on the integer pipes
+FP64_OPS_DX = 11
 
 
 def parse():
@@ -83,7 +86,7 @@ def parse():
     ap.add_argument("--epb", type=int, default=0,
                     help="fix the AX elements per CTA (1, 2 or 4; nek_set_ax_epb) instead of tuning")
     ap.add_argument("--ax", default="ff", choices=["fp64", "ff", "oz"],
-                    help="AX operator inside the solve: native FP64, FP64-accurate float-float, or FP64-accurate "
+                    help="AX operator inside the solve: FP64, FP64-accurate float-float, or FP64-accurate "
                          "with the contractions on the tensor cores (BF16 digit slices; even nx up to 10)")
     args = ap.parse_args()
     names = {"native", "sweep", "solve", "mixed", "learned", "batch", "lvec", "net"}
@@ -372,7 +375,8 @@ def ax_sweep(torch, nxs=(8, 10, 12, 16), reps=20, tune=False, elems=32):
             g = mesh.npts / t / 1e9
             res[name] = {"gdofs": g, "ms": t * 1e3, "gflops": g * perfmodel.ax_flops_per_point(nx),
                          "hbm_frac": g * 64 / hbm,
-                         "fp64_frac": g * perfmodel.ax_flops_per_point(nx) / 1e3 / FP64_PEAK_TFLOPS,
+                         "fp64_frac": g * (perfmodel.ax_flops_per_point(nx) if nx == 2 else 2 * FP64_OPS_DX if
+                                           name == "fp64" else 0) / 1e3 / FP64_PEAK_TFLOPS,
                          "epb": "2 persistent CTAs per SM" if name == "oz" else epb if epb is not None else
                          nekax.get_ax_epb(nekax.AX_FF if name == "ff" else nekax.AX_FP64, nx)}
         out[str(nx)] = res
@@ -614,8 +618,8 @@ def learned_block(torch, n_meshes=200, epochs=30, eval_elems=24):
 
 
 def native_fp64_block(torch, P, f, x, ws, iters, steps=3, tune=True):
-    """The headline solve with the native FP64 operator (nek_ax on the FP64 pipe): fixed-iteration rate and
-    its AX launches timed inside the solve."""
+    """The headline solve with the FP64 operator (nek_ax): fixed-iteration rate and its AX launches timed inside the
+    solve."""
     from paper_2011_04981_gb300 import nekax, perfmodel
 
     nx = P.nx
@@ -627,12 +631,12 @@ def native_fp64_block(torch, P, f, x, ws, iters, steps=3, tune=True):
     t_ax = out["ax"]["ms_per_launch"] / 1e3
     hbm, kind = peaks()
     flops = perfmodel.ax_flops_per_point(nx) * P.npts
-    out["ax"].update({"kernel": "k_ax_fp64<%d>" % nx, "tflops": flops / t_ax / 1e12,
-                      "fp64_pipe_frac": flops / t_ax / 1e12 / FP64_PEAK_TFLOPS,
+    out["ax"].update({"kernel": "k_ax_dx<%d>" % nx, "tflops": flops / t_ax / 1e12,
+                      "fp64_pipe_frac": 2 * FP64_OPS_DX * P.npts / t_ax / 1e12 / FP64_PEAK_TFLOPS,
                       "hbm_frac_64B": 64 * P.npts / t_ax / 1e9 / hbm,
                       "elements_per_cta": nekax.get_ax_epb(nekax.AX_FP64, nx)})
-    out["note"] = ("native FP64 (the paper's arithmetic); FP64 peak = 152 SM x 2 DFMA/clk x 2 flop x 2.07 GHz "
-                   "= %.4f TFLOP/s; HBM %s %.0f GB/s" % (FP64_PEAK_TFLOPS, kind, hbm))
+    out["note"] = ("FP64 operator (contractions in 58-bit block fixed point, G in FP64); FP64 peak = 152 SM x 2 DFMA/clk "
+                   "x 2 flop x 2.07 GHz = %.4f TFLOP/s; HBM %s %.0f GB/s" % (FP64_PEAK_TFLOPS, kind, hbm))
     return out
 
 
@@ -833,16 +837,17 @@ def run_native(args):
                "bytes_per_point": ax_bpp, "hbm_gbs": ax_bpp * pts / ax_t / 1e9,
                "hbm_frac": ax_bpp * pts / ax_t / 1e9 / hbm, "launches": ax_n,
                "share_of_step": ax_ms / 1e3 / t_dev, "elements_per_cta": ax_epb or "default"},
-        "roofline": ({"bound": "alu", "achieved": flops / ax_t / 1e12, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                      "frac": flops / ax_t / 1e12 / FP64_PEAK_TFLOPS, "traffic": traffic,
-                      "kernel": "k_ax_fp64<%d>" % nx,
-                      "note": "native FP64: DFMA-pipe bound; peak = 152 SM x 2 DFMA/clk x 2 x 2.07 GHz (nominal "
-                              "1.25 TFLOP/s); HBM %s peak %.0f GB/s" % (hbm_kind, hbm)}
+        "roofline": ({"bound": "alu", "achieved": 2 * FP64_OPS_DX * pts / ax_t / 1e12, "peak": FP64_PEAK_TFLOPS,
+                      "unit": "TFLOP/s", "frac": 2 * FP64_OPS_DX * pts / ax_t / 1e12 / FP64_PEAK_TFLOPS,
+                      "traffic": traffic, "kernel": "k_ax_dx<%d>" % nx,
+                      "note": "FP64 pipe by the product with G and the final sum (%d operations a point; the contractions "
+                              "are integer); peak = 152 SM x 2 DFMA/clk x 2 x 2.07 GHz (nominal 1.25 TFLOP/s); HBM %s "
+                              "peak %.0f GB/s" % (FP64_OPS_DX, hbm_kind, hbm)}
                      if args.ax == "fp64" else
                      {"bound": "hbm", "achieved": ax_bpp * pts / ax_t / 1e9, "peak": hbm, "unit": "GB/s",
                       "frac": ax_bpp * pts / ax_t / 1e9 / hbm, "traffic": traffic,
                       "kernel": ("k_ax_oz<%d, 2>" if args.ax == "oz" else
-                                 "k_ax_ffi<%d>" if nx in (10, 12) else "k_ax_ff<%d>") % nx,
+                                 "k_ax_fx<%d>" if nx >= 5 else "k_ax_ff<%d>") % nx,
                       "note": ("FP64-accurate AX (%s) with the fused x / direction update, 104 algorithmic "
                                "B/point (p in and out 16, r 8, minv 8, x in and out 16, G 48, w 8)"
                                % ("tensor-core digit slices" if args.ax == "oz" else "float-float") if fused_dir else

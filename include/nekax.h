@@ -53,7 +53,7 @@ typedef enum {
 
 /* Which AX operator a call uses. */
 typedef enum {
-    NEK_AX_FP64 = 0,      /* nek_ax: native FP64 */
+    NEK_AX_FP64 = 0,      /* nek_ax: FP64 */
     NEK_AX_FF = 1,        /* nek_ax_ff: FP64-accurate float-float on the FP32 pipes; needs Gff */
     NEK_AX_FF_ENERGY = 2, /* nek_ax_ff's element-energy form (nek_ax_ff_energy and the solves):
                              for nek_set_ax_epb / nek_get_ax_epb only */
@@ -95,11 +95,12 @@ nek_status nek_geom(int64_t nelt, int nx, const double* corners, double* G, void
 
 /* ------------------------------------------------------------------ AX ---
  * w = AX(u) on every element (Section II-B, Listing 1: ax, ax_e, local_grad3
- * and the transposed local_grad3_t), FP64 throughout.
+ * and the transposed local_grad3_t), FP64 in and out.
  *   nelt >= 0 elements (0 is a no-op), 2 <= nx <= 16;
  *   D: device, nx*nx; G: device, nelt*nx^3*6; u: device, in; w: device, out.
  *   u and w must not overlap.  Async on stream.
- * Native FP64 arithmetic on the double-precision pipe.
+ * To FP64 rounding: from nx = 3 on the contractions are summed in 58-bit block fixed point per line (integers; lines that
+ * are not finite or beyond 2^+-400 in FP64), the product with G in FP64; nx = 2 in FP64 throughout.
  */
 nek_status nek_ax(int64_t nelt, int nx, const double* D, const double* G, const double* u, double* w,
                   void* stream);

@@ -1,37 +1,22 @@
-// AX operator, native FP64 (Section II-B, Listing 1 of arXiv 2011.04981).
+// AX operator, FP64 (Section II-B, Listing 1 of arXiv 2011.04981): the dispatch over nx, the C entry point, and the kernel
+// of nx = 2.  nx >= 3 runs the line-pass kernel of nek_ax_dx.cuh.
 //
-// Per element the operator is
-//   ur = D_r u, us = D_s u, ut = D_t u             (local_grad3)
-//   [wr ws wt] = G [ur us ut]                        (the pointwise g product)
-//   w = D_r^T wr + D_s^T ws + D_t^T wt               (local_grad3_t)
-// with D_r acting on i, D_s on j and D_t on k of the [k][j][i] block.
-//
-// Kernel layout: a CTA owns EPB elements and has nx*nx*EPB threads; thread
-// (e, i, j) keeps the k-line u(i,j,:) and the t-results wt(i,j,:) in registers
-// and walks the k planes.  The u block of every element is staged in shared
-// memory once (one coalesced read of u: the FPGA design's single read of every
-// grid point of u becomes one pass through HBM here) so that the r- and
-// s-contractions read it from shared memory in their own order, which is what
-// the per-matmul reorder buffers of the FPGA design (Section III) achieve.
-// ws goes to shared memory as it is produced; wr is kept in registers until
-// every thread has finished reading u, then overwrites the u block, so each
-// element needs 2*nx^3 doubles of shared memory.  G is streamed from HBM exactly
-// once, w written exactly once.
+// nx = 2: a CTA owns EPB elements; thread (e, i, j) keeps the k-line u(i,j,:) and the t-results wt(i,j,:) in
+// registers and walks the k planes.  The u block of every element is staged in shared memory once (one coalesced read
+// of u: the FPGA design's single read of every grid point of u becomes one pass through HBM here) so that the r- and
+// s-contractions read it from shared memory in their own order, which is what the per-matmul reorder buffers of the FPGA
+// design (Section III) achieve.  ws goes to shared memory as it is produced; wr is kept in registers until every
+// thread has finished reading u, then overwrites the u block.  G is streamed from HBM exactly once, w written exactly once.
+// Lines of two points are too short for the line passes: 196608 elements take 72 us here, 86 in k_ax_dx; the latter
+// is faster from nx = 3 on (168 against 261 us).
 #include <algorithm>
 
+#include "nek_ax_dx.cuh"
 #include "nek_internal.h"
 
 namespace nek {
 
 namespace {
-
-// Elements per CTA for each nx, chosen so that nx*nx*EPB threads fill whole
-// warps as far as possible and several CTAs fit on one SM.
-constexpr int ax_epb(int nx)
-{
-    return nx == 2 ? 32 : nx == 3 ? 32 : nx == 4 ? 8 : nx == 5 ? 16 : nx == 6 ? 8 : nx == 7 ? 8 : nx == 8 ? 4
-         : nx == 9 ? 4 : nx == 10 ? 4 : nx == 11 ? 2 : nx == 12 ? 2 : nx == 13 ? 2 : 1;
-}
 
 template <int NX, int EPB>
 constexpr size_t ax_smem_bytes()
@@ -135,33 +120,11 @@ nek_status launch_ax_variant(int64_t nelt, const double* D, const double* G, con
     return check_launch();
 }
 
-template <int NX, int EPB>
-constexpr bool ax_fits()
+// The elements-per-CTA counts that are accepted: 1, 2 and 4; at nx = 16 1 and 2.
+constexpr bool ax_fits(int nx, int epb)
 {
-    return NX * NX * EPB <= 1024 && ax_smem_bytes<NX, EPB>() <= 227 * 1024;
-}
-
-template <int NX>
-nek_status launch_ax_nx(int epb, int64_t nelt, const double* D, const double* G, const double* u, double* w,
-                        cudaStream_t s)
-{
-    if (epb <= 0) epb = ax_epb(NX);
-    switch (epb) {
-        case 1:
-            if constexpr (ax_fits<NX, 1>()) return launch_ax_variant<NX, 1>(nelt, D, G, u, w, s);
-            break;
-        case 2:
-            if constexpr (ax_fits<NX, 2>()) return launch_ax_variant<NX, 2>(nelt, D, G, u, w, s);
-            break;
-        case 4:
-            if constexpr (ax_fits<NX, 4>()) return launch_ax_variant<NX, 4>(nelt, D, G, u, w, s);
-            break;
-        default:
-            break;
-    }
-    if constexpr (ax_epb(NX) != 1 && ax_epb(NX) != 2 && ax_epb(NX) != 4)
-        return launch_ax_variant<NX, ax_epb(NX)>(nelt, D, G, u, w, s);
-    return NEK_ERR_INVALID_ARG;
+    return (epb == 1 || epb == 2 || epb == 4) && nx * nx * epb <= 1024 &&
+           (nx * nx + 2 * epb * nx * nx * nx + 1) * 8 <= 227 * 1024;
 }
 
 }  // namespace
@@ -169,55 +132,22 @@ nek_status launch_ax_nx(int epb, int64_t nelt, const double* D, const double* G,
 nek_status launch_ax_fp64_epb(int epb, int64_t nelt, int nx, const double* D, const double* G, const double* u,
                               double* w, cudaStream_t s)
 {
-    switch (nx) {
-        case 2: return launch_ax_nx<2>(epb, nelt, D, G, u, w, s);
-        case 3: return launch_ax_nx<3>(epb, nelt, D, G, u, w, s);
-        case 4: return launch_ax_nx<4>(epb, nelt, D, G, u, w, s);
-        case 5: return launch_ax_nx<5>(epb, nelt, D, G, u, w, s);
-        case 6: return launch_ax_nx<6>(epb, nelt, D, G, u, w, s);
-        case 7: return launch_ax_nx<7>(epb, nelt, D, G, u, w, s);
-        case 8: return launch_ax_nx<8>(epb, nelt, D, G, u, w, s);
-        case 9: return launch_ax_nx<9>(epb, nelt, D, G, u, w, s);
-        case 10: return launch_ax_nx<10>(epb, nelt, D, G, u, w, s);
-        case 11: return launch_ax_nx<11>(epb, nelt, D, G, u, w, s);
-        case 12: return launch_ax_nx<12>(epb, nelt, D, G, u, w, s);
-        case 13: return launch_ax_nx<13>(epb, nelt, D, G, u, w, s);
-        case 14: return launch_ax_nx<14>(epb, nelt, D, G, u, w, s);
-        case 15: return launch_ax_nx<15>(epb, nelt, D, G, u, w, s);
-        case 16: return launch_ax_nx<16>(epb, nelt, D, G, u, w, s);
-        default: return NEK_ERR_UNSUPPORTED_NX;
+    if (nx < kMinNx || nx > kMaxNx) return NEK_ERR_UNSUPPORTED_NX;
+    if (epb > 0 && !ax_fits(nx, epb)) return NEK_ERR_INVALID_ARG;
+    if (nx == 2) {
+        switch (epb) {
+            case 1: return launch_ax_variant<2, 1>(nelt, D, G, u, w, s);
+            case 2: return launch_ax_variant<2, 2>(nelt, D, G, u, w, s);
+            case 4: return launch_ax_variant<2, 4>(nelt, D, G, u, w, s);
+            default: return launch_ax_variant<2, 32>(nelt, D, G, u, w, s);
+        }
     }
+    if (nx <= 7) return launch_ax_dx_a(nx, epb, nelt, D, G, u, w, s);
+    if (nx <= 11) return launch_ax_dx_b(nx, epb, nelt, D, G, u, w, s);
+    return launch_ax_dx_c(nx, epb, nelt, D, G, u, w, s);
 }
 
-namespace {
-template <int NX>
-bool ax_fits_rt(int epb)
-{
-    return (epb == 1 && ax_fits<NX, 1>()) || (epb == 2 && ax_fits<NX, 2>()) || (epb == 4 && ax_fits<NX, 4>());
-}
-}  // namespace
-
-bool ax_fp64_epb_fits(int nx, int epb)
-{
-    switch (nx) {
-        case 2: return ax_fits_rt<2>(epb);
-        case 3: return ax_fits_rt<3>(epb);
-        case 4: return ax_fits_rt<4>(epb);
-        case 5: return ax_fits_rt<5>(epb);
-        case 6: return ax_fits_rt<6>(epb);
-        case 7: return ax_fits_rt<7>(epb);
-        case 8: return ax_fits_rt<8>(epb);
-        case 9: return ax_fits_rt<9>(epb);
-        case 10: return ax_fits_rt<10>(epb);
-        case 11: return ax_fits_rt<11>(epb);
-        case 12: return ax_fits_rt<12>(epb);
-        case 13: return ax_fits_rt<13>(epb);
-        case 14: return ax_fits_rt<14>(epb);
-        case 15: return ax_fits_rt<15>(epb);
-        case 16: return ax_fits_rt<16>(epb);
-        default: return false;
-    }
-}
+bool ax_fp64_epb_fits(int nx, int epb) { return nx >= kMinNx && nx <= kMaxNx && ax_fits(nx, epb); }
 
 nek_status launch_ax_fp64(int64_t nelt, int nx, const double* D, const double* G, const double* u, double* w,
                           cudaStream_t s)

@@ -830,6 +830,64 @@ def test_ax_ff_non_finite_stays_in_its_element(nx, nelt):
     assert np.array_equal(w[rest], clean[rest]) and np.array_equal(ed[rest], ec[rest])
 
 
+@pytest.mark.parametrize("kind", ["gll", "general", "one entry off", "rows out of range"])
+@pytest.mark.parametrize("nx,nelt", [(2, 65), (3, 5), (3, 4001), (4, 2437), (5, 152), (5, 3001), (6, 153), (7, 1), (7, 2433), (8, 1300),
+                                     (9, 161), (10, 40), (11, 155), (12, 153), (13, 3), (14, 160), (15, 2), (16, 157)])
+def test_ax_fp64_any_matrix_and_any_range(nx, nelt, kind):
+    """The FP64 operator: D of the rule (folded rows), any D, one entry off, rows beyond the fixed point's range; element
+    counts on both sides of one per SM, ragged and above what is resident; elements that are zero, subnormal, tiny, huge
+    or not finite among the others; u at an address that is not 16-byte aligned.
+
+    Bound: a line sum is within 8 roundings of its largest value times the row's absolute sum, the oracle within nx + 4;
+    two such passes and G: (2 nx + 32) 2^-53 of 3 max(col sum) max(|G| row sum) max(row sum) max|u| of the element."""
+    rng = np.random.default_rng(40 + nx)
+    xi, rho, D = ref.gll(nx)
+    if kind == "general":
+        D = rng.uniform(-1, 1, size=(nx, nx)) * np.exp(rng.uniform(-3, 3, size=(nx, 1)))
+    elif kind == "one entry off":
+        D = D.copy()
+        D[nx // 2, 0] *= 1 + 2.0 ** -50
+    elif kind == "rows out of range":
+        D = D * 2.0 ** -450
+    base = min(nelt, 60)
+    mesh = inputs.box_mesh(base, 1, 1, nx, perturb=0.2, seed=nx)
+    G = ref.geom(mesh.corners, nx, xi, rho)[np.arange(nelt) % base]
+    u = rng.uniform(-1, 1, size=(nelt, nx ** 3)) * np.exp(rng.uniform(-20, 20, size=(nelt, 1)))
+    if nelt > 6 and kind != "rows out of range":
+        u[0] = 0.0
+        u[1] *= 1e-308 / np.abs(u[1]).max()
+        u[2] *= 1e200
+        u[3] *= 1e-250
+        u[4, nx] = np.inf
+        u[nelt - 1, nx ** 3 - 1] = np.nan
+    buf = torch.zeros(nelt * nx ** 3 + 1, dtype=torch.float64, device=DEV)
+    ut = buf[1:].view(nelt, nx ** 3)
+    ut.copy_(_t(u))
+    w = torch.full((nelt, nx ** 3), 7.0, dtype=torch.float64, device=DEV)
+    nekax.ax(nelt, nx, _t(D), _t(G), ut, w)
+    torch.cuda.synchronize()
+    w, wr = w.cpu().numpy(), ref.ax(D, G, u)
+    fin = np.isfinite(wr)
+    assert np.array_equal(np.isfinite(w), fin)
+    a, g = np.abs(D), np.abs(G).reshape(nelt, nx ** 3, 6)
+    rows = np.stack([g[..., [0, 1, 2]].sum(-1), g[..., [1, 3, 4]].sum(-1), g[..., [2, 4, 5]].sum(-1)], -1).max((1, 2))
+    um = np.where(np.isfinite(u), np.abs(u), 0.0).max(1)
+    bound = (2 * nx + 32) * 2.0 ** -53 * 3 * a.sum(0).max() * rows * a.sum(1).max() * um + nx ** 3 * 2.0 ** -1060
+    err = np.where(fin, np.abs(np.where(fin, w, 0) - np.where(fin, wr, 0)), 0.0).max(1)
+    assert np.all(err <= bound), np.max(err / bound)
+    ones = np.where(np.isfinite(u).all(1))[0]
+    for epb in (1, 2, 4):  # the grouping changes no bit
+        if nekax.load().nek_set_ax_epb(int(nekax.AX_FP64), nx, epb) != nekax.OK:
+            continue
+        try:
+            w2 = torch.full((nelt, nx ** 3), 7.0, dtype=torch.float64, device=DEV)
+            nekax.ax(nelt, nx, _t(D), _t(G), ut, w2)
+            torch.cuda.synchronize()
+        finally:
+            nekax.load().nek_set_ax_epb(int(nekax.AX_FP64), nx, 0)
+        assert np.array_equal(w2.cpu().numpy()[ones], w[ones])
+
+
 def test_batch_skips_finished_elements_beyond_the_resident_ctas():
     """Problems of more elements than the resident CTAs hold, one of them finished from the start (f = 0): the CTAs
     pass over its elements and the others' iterates are those of a batch without it."""
