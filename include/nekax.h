@@ -553,7 +553,7 @@ nek_status nek_fcg_solve(const nek_gs* gs, int64_t nelt, int nx, const double* D
 size_t nek_cg_workspace_bytes(int64_t nelt, int nx, int need_minv);
 
 typedef struct {
-    int check_every;     /* residual read-back period in iterations (>=1; default 1) */
+    int check_every;     /* residual read-back period in iterations (>=1; default 1); the result does not depend on it */
     int time_ax;         /* nonzero: record CUDA events around every AX launch */
     double ax_ms_total;  /* out: summed AX kernel time when time_ax */
     int ax_launches;     /* out: number of AX launches */

@@ -87,12 +87,17 @@ __device__ __forceinline__ double dx_ldexp(long long z, int x)
     return __hiloint2double((int)((int)(g >> 32) >= 0 ? 0u : hi | ((unsigned)sg & 0x80000000u)), (int)(unsigned)m);
 }
 
-// Fills t[0] (M = D) and t[1] (M = D^T), in integers (an FP64 chain here would be a third of the time of a call on few
+// Copies the matrix Dg to D, finds out whether it is symmetric as above, and fills t[0] (M = D) and t[1] (M = D^T), in integers (an FP64 chain here would be a third of the time of a call on few
 // elements).  Returns whether a row's absolute sum is outside kDxRange; the tables are then not to be used.
 template <int NX>
-__device__ __forceinline__ bool dx_build(const double* D, DxTab<NX>* t, int tid, int nt)
+__device__ __forceinline__ bool dx_build(const double* __restrict__ Dg, double* D, DxTab<NX>* t, int tid, int nt, bool& sym)
 {
-    constexpr int HE = DxTab<NX>::HE;
+    constexpr int HE = DxTab<NX>::HE, N2 = NX * NX;
+    for (int q = tid; q < N2; q += nt) D[q] = Dg[q];
+    __syncthreads();
+    bool asym = false;
+    for (int q = tid; q < N2; q += nt) asym = asym || D[q] != -D[N2 - 1 - q];
+    sym = !__syncthreads_or(asym);
     auto entry = [&](int m, int i, int l) { return m ? D[l * NX + i] : D[i * NX + l]; };
     bool bad = false;
     for (int r = tid; r < 2 * NX; r += nt) {
@@ -259,6 +264,55 @@ __device__ __forceinline__ void dx_lines(const double* const (&src)[LPT], double
     }
 }
 
+// A thread's lines (line L of an element: direction L / nx^2, line L % nx^2 of it), t the thread's number within its
+// element, slot the element's place; a thread whose last line would be past the end repeats its first.
+template <int NX, int LPT>
+struct DxLines {
+    const double *u[LPT], *in[LPT];  // phase 1 and phase 2 inputs
+    double* a[LPT];
+    int str[LPT];
+    unsigned sgn[LPT];
+
+    __device__ __forceinline__ DxLines(double* U, double* A0, int astride, int slot, int t, bool sym)
+    {
+        using Grid = FxGrid<NX>;
+        constexpr int N2 = NX * NX, TPE = dx_tpe(NX, LPT);
+#pragma unroll
+        for (int q = 0; q < LPT; q++) {
+            const int L = t + q * TPE < 3 * N2 ? t + q * TPE : t;
+            const int d = L / N2, c = L - d * N2, y = c / NX, x = c - y * NX;
+            int base = slot + (d == 0 ? x * Grid::ROW + y * Grid::PLANE : x + y * (d == 1 ? Grid::PLANE : Grid::ROW));
+            str[q] = d == 0 ? 1 : d == 1 ? Grid::ROW : Grid::PLANE;
+            sgn[q] = 0u;
+            if (Grid::REV != 0 && d == 0 && sym && (t / (Grid::REV ? Grid::REV : 1)) & 1) {
+                base += NX - 1;
+                str[q] = -1;
+                sgn[q] = 0x80000000u;
+            }
+            u[q] = U + base;
+            a[q] = A0 + d * astride + base;
+            in[q] = a[q];
+        }
+    }
+};
+
+// [wr ws wt] = G [ur us ut] in place on the thread's points t, t + TPE, ... of an element; Ge: its factors.
+template <int NX, int TPE>
+__device__ __forceinline__ void dx_geom(const double* __restrict__ Ge, double* const (&At)[3], int t)
+{
+    using Grid = FxGrid<NX>;
+    const double2* gp = reinterpret_cast<const double2*>(Ge + 6 * t);
+#pragma unroll 3
+    for (int p = t; p < NX * NX * NX; p += TPE, gp += 3 * TPE) {
+        const int a = Grid::at(p) - Grid::at(t);
+        const double2 g01 = __ldg(gp), g23 = __ldg(gp + 1), g45 = __ldg(gp + 2);
+        const double ar = At[0][a], as = At[1][a], at = At[2][a];
+        At[0][a] = fma(g01.x, ar, fma(g01.y, as, g23.x * at));
+        At[1][a] = fma(g01.y, ar, fma(g23.y, as, g45.x * at));
+        At[2][a] = fma(g23.x, ar, fma(g45.x, as, g45.y * at));
+    }
+}
+
 template <int NX, int EPB, int LPT>
 constexpr int dx_min_blocks()
 {
@@ -274,7 +328,7 @@ __global__ void __launch_bounds__(dx_threads(NX, EPB, LPT), (dx_min_blocks<NX, E
             double* __restrict__ w)
 {
     using Grid = FxGrid<NX>;
-    constexpr int NP = Grid::SIZE, N2 = NX * NX, N3 = NX * NX * NX;
+    constexpr int NP = Grid::SIZE, N3 = NX * NX * NX;
     constexpr int TPE = dx_tpe(NX, LPT), NT = dx_threads(NX, EPB, LPT);
     constexpr int B = (N3 + TPE - 1) / TPE;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -303,35 +357,10 @@ __global__ void __launch_bounds__(dx_threads(NX, EPB, LPT), (dx_min_blocks<NX, E
     fetch(e0);
 
     // ---- the matrix tables, once per CTA
-    for (int q = tid; q < N2; q += NT) S.D[q] = D[q];
-    __syncthreads();
-    bool asym = false;
-    for (int q = tid; q < N2; q += NT) asym = asym || S.D[q] != -S.D[N2 - 1 - q];
-    const bool sym = !__syncthreads_or(asym);
-    const bool bad = dx_build<NX>(S.D, S.tab, tid, NT);
+    bool sym;
+    const bool bad = dx_build<NX>(D, S.D, S.tab, tid, NT, sym);
 
-    // this thread's lines (line L: direction L / N2, line L % N2 of it), all of element el; a thread whose last
-    // line would be past the end repeats its first
-    const double *src1[LPT], *src2[LPT];
-    double* dstA[LPT];
-    int str[LPT];
-    unsigned sgn[LPT];
-#pragma unroll
-    for (int q = 0; q < LPT; q++) {
-        const int L = t + q * TPE < 3 * N2 ? t + q * TPE : t;
-        const int d = L / N2, c = L - d * N2, b = c / NX, a = c - b * NX;
-        int base = slot + (d == 0 ? a * Grid::ROW + b * Grid::PLANE : a + b * (d == 1 ? Grid::PLANE : Grid::ROW));
-        str[q] = d == 0 ? 1 : d == 1 ? Grid::ROW : Grid::PLANE;
-        sgn[q] = 0u;
-        if (Grid::REV != 0 && d == 0 && sym && (t / (Grid::REV ? Grid::REV : 1)) & 1) {
-            base += NX - 1;
-            str[q] = -1;
-            sgn[q] = 0x80000000u;
-        }
-        src1[q] = S.U + base;
-        dstA[q] = S.A[d] + base;
-        src2[q] = dstA[q];
-    }
+    DxLines<NX, LPT> ln(S.U, S.A[0], EPB * NP, slot, t, sym);
     double* At[3];
 #pragma unroll
     for (int d = 0; d < 3; d++) At[d] = S.A[d] + slot + Grid::at(t);
@@ -345,23 +374,12 @@ __global__ void __launch_bounds__(dx_threads(NX, EPB, LPT), (dx_min_blocks<NX, E
                          : "memory");
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        if (active) dx_lines<NX, false, LPT>(src1, dstA, str, sgn, S.tab[0], S.D, sym, bad);
+        if (active) dx_lines<NX, false, LPT>(ln.u, ln.a, ln.str, ln.sgn, S.tab[0], S.D, sym, bad);
         __syncthreads();
         if (e0 + step < nelt) fetch(e0 + step);  // U is free: every line has been read
-        if (active) {
-            const double2* gp = reinterpret_cast<const double2*>(G + (ef + t) * 6);
-#pragma unroll 3
-            for (int p = t; p < N3; p += TPE, gp += 3 * TPE) {
-                const int a = Grid::at(p) - Grid::at(t);
-                const double2 g01 = __ldg(gp), g23 = __ldg(gp + 1), g45 = __ldg(gp + 2);
-                const double ar = At[0][a], as = At[1][a], at = At[2][a];
-                At[0][a] = fma(g01.x, ar, fma(g01.y, as, g23.x * at));
-                At[1][a] = fma(g01.y, ar, fma(g23.y, as, g45.x * at));
-                At[2][a] = fma(g23.x, ar, fma(g45.x, as, g45.y * at));
-            }
-        }
+        if (active) dx_geom<NX, TPE>(G + ef * 6, At, t);
         __syncthreads();
-        if (active) dx_lines<NX, true, LPT>(src2, dstA, str, sgn, S.tab[1], S.D, sym, bad);
+        if (active) dx_lines<NX, true, LPT>(ln.in, ln.a, ln.str, ln.sgn, S.tab[1], S.D, sym, bad);
         __syncthreads();
         if (active) {
             double* we = w + ef + t;

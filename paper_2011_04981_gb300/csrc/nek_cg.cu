@@ -233,8 +233,12 @@ nek_status nek_cg_solve_ex(const nek_gs* gs, int64_t nelt, int nx, const double*
                    : ax_impl == NEK_AX_OZ ? launch_ax_oz(nelt, nx, D, Gff, p, w, ss, ed, dir)
                                           : launch_ax_fp64(nelt, nx, D, G, p, w, ss);
         };
-        st = pcg::run<double>(gs, n, gs->d_c, mask, mv, f, x, b, tol_rel, max_iter, check_every, time_ax, ax, s,
-                              &res, flags, energies ? &ee : nullptr);
+        bool ran = false;
+        if (ax_impl == NEK_AX_FP64 && !time_ax)
+            st = pcg::run_small(gs, nelt, nx, D, G, mask, mv, flags, f, x, b, edot, tol_rel, max_iter, s, &res, ran);
+        if (!ran && st == NEK_OK)
+            st = pcg::run<double>(gs, n, gs->d_c, mask, mv, f, x, b, tol_rel, max_iter, check_every, time_ax, ax, s,
+                                  &res, flags, energies ? &ee : nullptr);
         if (iters_out) *iters_out = res.iters;
         if (relres_out) *relres_out = res.relres;
         if (opts) {

@@ -427,26 +427,30 @@ __global__ void __launch_bounds__(NT) k_update(int64_t n, const V* __restrict__ 
     write_two_partials<NT>(arr, arz, parts, sh);
 }
 
+// The residual test and beta, from the sums rr and rz; one thread.
+__device__ __forceinline__ void set_beta(double rr, double rz, Scalars* sc)
+{
+    sc->rr = rr;
+    sc->relres = sqrt(rr) / sc->bnorm;
+    if (!isfinite(sc->relres) || !isfinite(rz)) {
+        sc->status = NEK_ERR_BREAKDOWN;
+        sc->iters = sc->it;
+    } else if (sc->tol > 0.0 && sc->relres <= sc->tol) {
+        sc->done = 1;
+        sc->iters = sc->it;
+    } else {
+        sc->beta = rz / sc->rz;
+        sc->rz = rz;
+    }
+}
+
 __global__ void __launch_bounds__(NT) k_beta(const double* __restrict__ parts, int nb, Scalars* sc)
 {
     __shared__ double sh[2 * NT];
     if (halted(sc)) return;
     double rr, rz;
     sum_two_partials<NT>(parts, nb, sh, rr, rz);
-    if (threadIdx.x == 0) {
-        sc->rr = rr;
-        sc->relres = sqrt(rr) / sc->bnorm;
-        if (!isfinite(sc->relres) || !isfinite(rz)) {
-            sc->status = NEK_ERR_BREAKDOWN;
-            sc->iters = sc->it;
-        } else if (sc->tol > 0.0 && sc->relres <= sc->tol) {
-            sc->done = 1;
-            sc->iters = sc->it;
-        } else {
-            sc->beta = rz / sc->rz;
-            sc->rz = rz;
-        }
-    }
+    if (threadIdx.x == 0) set_beta(rr, rz, sc);
 }
 
 // x += alpha p (old p) while xpend is set; then, when the iteration goes on and
@@ -533,6 +537,21 @@ inline nek_status build_flags(const nek_gs* gs, int64_t n, const uint8_t* mask, 
     return check_launch();
 }
 
+// The iteration count, residual norm and status of a finished solve from its scalars.
+inline nek_status result_of(const Scalars& h, double tol, Result* res)
+{
+    res->iters = (h.done || h.status != NEK_OK) ? h.iters : h.it;
+    res->relres = h.relres;
+    if (h.status != NEK_OK) return static_cast<nek_status>(h.status);
+    return tol > 0.0 && !h.done ? NEK_ERR_NOT_CONVERGED : NEK_OK;
+}
+
+// The FP64 solve of few elements in one launch (nek_cg_small.cu): ran is false, and nothing but the buffers written,
+// where the elements or the iterations are too many for it.  edot: nelt doubles of scratch; the rest as run.
+nek_status run_small(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G, const uint8_t* mask,
+                     const double* minv, const uint8_t* flags, const double* f, double* x, const Buffers<double>& b,
+                     double* edot, double tol, int max_iter, cudaStream_t s, Result* res, bool& ran);
+
 // Runs PCG from x = 0.  `ax(p, w, edot, dir, stream)` applies the element
 // operator, which gs then sums over shared nodes; with gs null, ax applies the
 // assembled operator itself.  edot is ee->edot on the element-energy path (ee
@@ -607,12 +626,7 @@ nek_status run(const nek_gs* gs, int64_t n, const V* c, const uint8_t* mask, con
         res->ax_ms = tot;
         res->ax_timed = nt;
     }
-    res->iters = (h.done || h.status != NEK_OK) ? h.iters : h.it;
-    res->relres = h.relres;
-    if (h.status != NEK_OK)
-        st = static_cast<nek_status>(h.status);
-    else if (tol > 0.0 && !h.done)
-        st = NEK_ERR_NOT_CONVERGED;
+    st = result_of(h, tol, res);
 done:
     for (auto& e : ev)
         if (e) cudaEventDestroy(e);

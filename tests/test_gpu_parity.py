@@ -888,6 +888,46 @@ def test_ax_fp64_any_matrix_and_any_range(nx, nelt, kind):
         assert np.array_equal(w2.cpu().numpy()[ones], w[ones])
 
 
+@pytest.mark.parametrize("dims,nx", [((1, 1, 1), 4), ((3, 2, 2), 4), ((13, 9, 9), 4), ((2, 1, 1), 5), ((5, 4, 3), 6), ((3, 3, 2), 7),
+                                     ((1, 1, 1), 8), ((8, 19, 3), 8), ((3, 3, 3), 9), ((4, 3, 3), 10), ((3, 2, 1), 11),
+                                     ((8, 19, 1), 12), ((2, 2, 2), 13), ((3, 2, 2), 14), ((2, 1, 2), 15), ((2, 2, 1), 16)])
+def test_cg_of_few_elements_in_one_launch(dims, nx):
+    """The FP64 solve in one launch, up to the most elements it takes, against the loop of launches (which timing the
+    operator selects): the same operations on every point, sums in another order.  A fixed number of iterations: equal
+    counts, iterates within the 1e-9 that any two orders of the solve's sums are held to.  To a tolerance (hundreds of
+    iterations amplify the order of the sums: the loop's own count moves by one from operator to operator): the oracle's
+    residual."""
+    mesh = inputs.box_mesh(*dims, nx, perturb=0.1, seed=nx)
+    P = DeviceProblem(mesh, DEV)
+    fh = inputs.random_global_field(mesh, seed=3)
+    f = _t(fh)
+    x1, x2 = torch.full_like(f, 5.0), torch.full_like(f, 5.0)
+    for kw in (dict(tol=0.0, max_iter=12), dict(tol=1e-7, max_iter=3)):
+        a = P.cg(f, x1, **kw)
+        b = P.cg(f, x2, time_ax=True, **kw)
+        assert a["kernel_launches"] <= 10 and (a["status"], a["iters"]) == (b["status"], b["iters"])
+        assert abs(a["relres"] - b["relres"]) <= 1e-6 * b["relres"]
+        assert float((x1 - x2).abs().max()) <= 1e-9 * float(x2.abs().max())
+    a = P.cg(f, x1, tol=1e-7, max_iter=3000)
+    assert a["kernel_launches"] <= 10 and a["status"] == nekax.OK and a["relres"] <= 1e-7
+    assert ref.Problem(mesh).residual(fh, x1.cpu().numpy().reshape(mesh.nelt, -1)) <= 1e-7 * 1.001
+    assert P.cg(torch.zeros_like(f), x1, tol=1e-7)["iters"] == 0 and torch.all(x1 == 0)
+    assert P.cg(f, x1, tol=1e-7, max_iter=0)["iters"] == 0 and torch.all(x1 == 0)
+    g = f.clone()
+    g.view(-1)[int(torch.nonzero(P.mask.view(-1))[0])] = float("nan")  # on a free node
+    a, b = P.cg(g, x1, tol=1e-7), P.cg(g, x2, tol=1e-7, time_ax=True)
+    assert (a["status"], a["iters"]) == (b["status"], b["iters"]) and a["status"] != nekax.OK
+
+
+def test_cg_of_more_elements_than_one_launch_takes():
+    mesh = inputs.box_mesh(9, 17, 1, 12, perturb=0.1, seed=1)
+    P = DeviceProblem(mesh, DEV)
+    f = _t(inputs.random_global_field(mesh, seed=3))
+    x = torch.empty_like(f)
+    r = P.cg(f, x, tol=0.0, max_iter=5)
+    assert r["iters"] == 5 and r["kernel_launches"] > 30
+
+
 def test_batch_skips_finished_elements_beyond_the_resident_ctas():
     """Problems of more elements than the resident CTAs hold, one of them finished from the start (f = 0): the CTAs
     pass over its elements and the others' iterates are those of a batch without it."""
