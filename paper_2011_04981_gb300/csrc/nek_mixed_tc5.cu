@@ -24,6 +24,13 @@
 // with that solve's own FP32 operations; the operator is applied to the new p),
 // which takes the solve's separate x / direction pass over the vectors away.
 //
+// What bounds it (nx = 10, 4096 elements, FP16, with the direction update; launch list, cold cache): latency, the chain
+// of six block barriers, two MMA round trips and the memory reads of an element; the shared-memory path is 56 % busy, issue
+// 32 %, DRAM 40 %.  The reads are taken out of the chain: an element's G words are in registers from its start, its inputs
+// from the second phase of the element before, its u stays in shared memory for the energies.  That costs registers, and 4
+// CTAs an SM that do not wait beat more that do: 49.8 us without (7 CTAs), 46.5 with G early only, 49.2 / 46.0 / 44.2 with
+// both at 6 / 5 / 4 CTAs.
+//
 // Every wait on the mbarrier is bounded (~2 s of global time); a wait that
 // runs out writes NaN into the CTA's remaining outputs, waits once more for its
 // MMAs, frees its tensor memory and returns.
@@ -80,12 +87,18 @@ constexpr size_t tc5_x_bytes()
 {
     return (sizeof(float) * 3 * (size_t)NX * NX * NX + 15) & ~size_t(15);
 }
-// The point arrays (the element's u, then ur us ut, wr ws wt, the parts of w), A [3], B [2], then 64 bytes
-// of scalars and 32 of per-warp energies: 25.4 KB at nx = 10, so that 8 CTAs fit on an SM.
+// The element's u, rounded up to 16 bytes.
+template <int NX>
+constexpr size_t tc5_u_bytes()
+{
+    return (sizeof(float) * (size_t)NX * NX * NX + 15) & ~size_t(15);
+}
+// The point arrays (ur us ut, wr ws wt, the parts of w), u, A [3], B [2], then 64 bytes of scalars and 32 of per-warp
+// energies: 29.4 KB at nx = 10.
 template <int NX>
 constexpr size_t tc5_smem_bytes()
 {
-    return 3 * kABytes + 2 * kBBytes + tc5_x_bytes<NX>() + 96;
+    return 3 * kABytes + 2 * kBBytes + tc5_x_bytes<NX>() + tc5_u_bytes<NX>() + 96;
 }
 
 __device__ int g_lowp_tc5_timeout = 0;
@@ -125,16 +138,14 @@ __device__ __forceinline__ float pow2_up(float m)
     return ldexpf(1.f, f == 0.5f ? e - 1 : e);
 }
 
-// Six G values of point p as floats (12 bytes at a 4-byte aligned address).
+// Six G values of a point (three words of two) as floats.
 template <class S>
-__device__ __forceinline__ void g_load(const S* __restrict__ g, float (&v)[6])
+__device__ __forceinline__ void g_values(const unsigned (&t)[3], float (&v)[6])
 {
-    const unsigned* g4 = reinterpret_cast<const unsigned*>(g);
 #pragma unroll
     for (int q = 0; q < 3; q++) {
-        const unsigned t = __ldg(g4 + q);
-        v[2 * q] = Lp5<S>::from_bits(static_cast<unsigned short>(t & 0xffffu));
-        v[2 * q + 1] = Lp5<S>::from_bits(static_cast<unsigned short>(t >> 16));
+        v[2 * q] = Lp5<S>::from_bits(static_cast<unsigned short>(t[q] & 0xffffu));
+        v[2 * q + 1] = Lp5<S>::from_bits(static_cast<unsigned short>(t[q] >> 16));
     }
 }
 
@@ -149,7 +160,7 @@ __device__ __forceinline__ void issue3(uint32_t tmem, uint32_t a_base, uint32_t 
 }
 
 template <class S, int NX, int MODE>
-__global__ void __launch_bounds__(kT5, MODE == kLpDir ? 6 : 4)
+__global__ void __launch_bounds__(kT5, 4)
     k_ax_lowp_tc5(int64_t nelt, const double* __restrict__ D, const S* __restrict__ Glp,
                   const float* __restrict__ gscale, const float* __restrict__ u, float* __restrict__ w,
                   double* __restrict__ edot, DirUpdateF dir, long long wait_ns)
@@ -160,9 +171,9 @@ __global__ void __launch_bounds__(kT5, MODE == kLpDir ? 6 : 4)
     unsigned char* A = lp5_raw;                                        // [3][kABytes]
     unsigned char* B1 = A + 3 * kABytes;                               // rnd(D)
     unsigned char* B2 = B1 + kBBytes;                                  // rnd(D)^T
-    float* X = reinterpret_cast<float*>(B2 + kBBytes);                // [3][N3] u; ur us ut; wr ws wt; w parts
-    float* sU = X;                                                     // the element's u until the first readout
-    unsigned char* tail = B2 + kBBytes + tc5_x_bytes<NX>();            // 16-byte aligned
+    float* X = reinterpret_cast<float*>(B2 + kBBytes);                // [3][N3] ur us ut; wr ws wt; w parts
+    float* sU = reinterpret_cast<float*>(B2 + kBBytes + tc5_x_bytes<NX>());  // the element's u
+    unsigned char* tail = reinterpret_cast<unsigned char*>(sU) + tc5_u_bytes<NX>();  // 16-byte aligned
     unsigned long long* mbar_p = reinterpret_cast<unsigned long long*>(tail);
     uint32_t* tmem_p = reinterpret_cast<uint32_t*>(tail + 8);
     float* red = reinterpret_cast<float*>(tail + 16);                  // [4]
@@ -203,6 +214,29 @@ __global__ void __launch_bounds__(kT5, MODE == kLpDir ? 6 : 4)
         beta = (float)dir.sc->beta;
     }
 
+    // This thread's points tid, tid + 128, ... of an element: their inputs (u; with the direction update p, r, minv, x) are
+    // loaded while the element before is in its second phase, so that no phase starts by waiting for memory.
+    constexpr int B = (N3 + kT5 - 1) / kT5, NIN = MODE == kLpDir ? 4 : 1, kG = B < 8 ? B : 8;
+    constexpr bool kCarry = B <= 8;
+    float in[NIN][B];
+    auto has = [&](int k) { return k < B - 1 || tid + k * kT5 < N3; };
+    auto load_in = [&](int64_t el) {
+        const int64_t o = el * N3 + tid;
+#pragma unroll
+        for (int k = 0; k < B; k++) {
+            if (has(k)) {
+                if constexpr (MODE == kLpDir) {
+                    in[0][k] = dir.p[o + k * kT5];
+                    in[1][k] = __ldg(dir.r + o + k * kT5);
+                    in[2][k] = __ldg(dir.minv + o + k * kT5);
+                    in[3][k] = dx ? dir.x[o + k * kT5] : 0.f;
+                } else {
+                    in[0][k] = __ldg(u + o + k * kT5);
+                }
+            }
+        }
+    };
+    if (kCarry && (int64_t)blockIdx.x < nelt) load_in(blockIdx.x);
     for (int64_t e = blockIdx.x; e < nelt; e += gridDim.x) {
         // the next element's inputs and G into L2 while this one is processed
         if (e + gridDim.x < nelt) {
@@ -224,45 +258,39 @@ __global__ void __launch_bounds__(kT5, MODE == kLpDir ? 6 : 4)
         }
         // ---- u (with the direction update: the new p) into shared memory, the element's scale s_u
         float mx = 0.f;
+        if (!kCarry) load_in(e);
         if constexpr (MODE == kLpDir) {
-            float* pe = dir.p + e * N3;
-            float* xe = dir.x + e * N3;
-            const float* re = dir.r + e * N3;
-            const float* me = dir.minv + e * N3;
-            constexpr int KB = 4;  // points per batch: a batch's loads are issued before its stores
-            for (int q0 = tid; q0 < N3; q0 += KB * kT5) {
-                float po[KB], rv[KB], mv[KB], xv[KB];
+            float* pe = dir.p + e * N3 + tid;
+            float* xe = dir.x + e * N3 + tid;
 #pragma unroll
-                for (int k = 0; k < KB; k++) {
-                    const int q = q0 + k * kT5 < N3 ? q0 + k * kT5 : q0;
-                    po[k] = pe[q];
-                    rv[k] = __ldg(re + q);
-                    mv[k] = __ldg(me + q);
-                    xv[k] = dx ? xe[q] : 0.f;
-                }
-#pragma unroll
-                for (int k = 0; k < KB; k++) {
-                    const int q = q0 + k * kT5;
-                    if (q < N3) {
-                        if (dx) xe[q] = fmaf(alpha, po[k], xv[k]);
-                        float v = po[k];
-                        if (dp) {
-                            v = fmaf(beta, po[k], mv[k] * rv[k]);
-                            pe[q] = v;
-                        }
-                        sU[q] = v;
-                        mx = fmaxf(mx, fabsf(v));
+            for (int k = 0; k < B; k++) {
+                if (has(k)) {
+                    if (dx) xe[k * kT5] = fmaf(alpha, in[0][k], in[3][k]);
+                    float v = in[0][k];
+                    if (dp) {
+                        v = fmaf(beta, v, in[2][k] * in[1][k]);
+                        pe[k * kT5] = v;
                     }
+                    sU[tid + k * kT5] = v;
+                    mx = fmaxf(mx, fabsf(v));
                 }
             }
         } else {
-            const float* ue = u + e * N3;
-            for (int q = tid; q < N3; q += kT5) {
-                const float v = __ldg(ue + q);
-                sU[q] = v;
-                mx = fmaxf(mx, fabsf(v));
+#pragma unroll
+            for (int k = 0; k < B; k++) {
+                if (has(k)) {
+                    sU[tid + k * kT5] = in[0][k];
+                    mx = fmaxf(mx, fabsf(in[0][k]));
+                }
             }
         }
+        // the first kG of this thread's points' geometric factors, in flight until phase 1 is read out
+        unsigned gr[kG][3];
+        const unsigned* Ge = reinterpret_cast<const unsigned*>(Glp + e * (int64_t)N3 * 6) + 3 * tid;
+#pragma unroll
+        for (int k = 0; k < kG; k++)
+#pragma unroll
+            for (int q = 0; q < 3; q++) gr[k][q] = has(k) ? __ldg(Ge + 3 * k * kT5 + q) : 0u;
         const float su = pow2_up(cta_max(mx, red));
         const float inv = 1.f / su;  // a power of two: exact
         // ---- A rows: this thread's three lines of rnd(u / s_u)
@@ -310,14 +338,20 @@ __global__ void __launch_bounds__(kT5, MODE == kLpDir ? 6 : 4)
         __syncthreads();
         // ---- wr, ws, wt = rnd(G_q [ur us ut]) in FP32, in place
         {
-            const S* Ge = Glp + e * (int64_t)N3 * 6;
-            for (int p = tid; p < N3; p += kT5) {
-                const float ar = X[p], as = X[N3 + p], at = X[2 * N3 + p];
-                float g[6];
-                g_load<S>(Ge + 6 * p, g);
-                X[p] = Lp5<S>::from_bits(Lp5<S>::bits(fmaf(g[0], ar, fmaf(g[1], as, g[2] * at))));
-                X[N3 + p] = Lp5<S>::from_bits(Lp5<S>::bits(fmaf(g[1], ar, fmaf(g[3], as, g[4] * at))));
-                X[2 * N3 + p] = Lp5<S>::from_bits(Lp5<S>::bits(fmaf(g[2], ar, fmaf(g[4], as, g[5] * at))));
+#pragma unroll
+            for (int k = 0; k < B; k++) {
+                if (has(k)) {
+                    const int p = tid + k * kT5;
+                    const float ar = X[p], as = X[N3 + p], at = X[2 * N3 + p];
+                    unsigned t[3];
+#pragma unroll
+                    for (int q = 0; q < 3; q++) t[q] = k < kG ? gr[k < kG ? k : 0][q] : __ldg(Ge + 3 * k * kT5 + q);
+                    float g[6];
+                    g_values<S>(t, g);
+                    X[p] = Lp5<S>::from_bits(Lp5<S>::bits(fmaf(g[0], ar, fmaf(g[1], as, g[2] * at))));
+                    X[N3 + p] = Lp5<S>::from_bits(Lp5<S>::bits(fmaf(g[1], ar, fmaf(g[3], as, g[4] * at))));
+                    X[2 * N3 + p] = Lp5<S>::from_bits(Lp5<S>::bits(fmaf(g[2], ar, fmaf(g[4], as, g[5] * at))));
+                }
             }
         }
         __syncthreads();
@@ -342,6 +376,7 @@ __global__ void __launch_bounds__(kT5, MODE == kLpDir ? 6 : 4)
             issue3(tmem, a_base, b2, IDESC, mbar);
             __syncwarp();
         }
+        if (kCarry && e + gridDim.x < nelt) load_in(e + gridDim.x);
         if (tid == 0) *flag = tc5::mbar_wait_bounded(mbar, parity, wait_ns, kHint5) ? 0 : 1;
         __syncthreads();
         if (*flag) goto timed_out;
@@ -372,9 +407,7 @@ __global__ void __launch_bounds__(kT5, MODE == kLpDir ? 6 : 4)
             for (int p = tid; p < N3; p += kT5) {
                 const float wv = ((X[p] + X[N3 + p]) + X[2 * N3 + p]) * scale;
                 we[p] = wv;
-                // the input at p: with the direction update the p this thread wrote above (a plain load)
-                if constexpr (MODE == kLpDir) energy = fmaf(dir.p[e * N3 + p], wv, energy);
-                if constexpr (MODE == kLpEnergy) energy = fmaf(__ldg(u + e * N3 + p), wv, energy);
+                if constexpr (MODE != kLpPlain) energy = fmaf(sU[p], wv, energy);
             }
             if constexpr (MODE != kLpPlain) {
                 double t = (double)energy;
