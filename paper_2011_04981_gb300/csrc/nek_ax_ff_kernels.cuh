@@ -505,8 +505,11 @@ nek_status launch_ax_ff_kernel(int64_t nelt, const double* D, const float* Gff, 
         nek_status st = ensure_dyn_smem(k_ax_fx<NX, C, MODE>, smem, configured);
         if (st != NEK_OK) return st;
         const int64_t groups = (nelt + C - 1) / C, resident = kSMs * fx_min_blocks<NX, C>();
-        k_ax_fx<NX, C, MODE><<<(unsigned)(groups < resident ? groups : resident), fx_threads(NX, C), smem, s>>>(
-            nelt, D, G4, u, w, l2g, eprob, pdone, edot, d);
+        const int grid = (int)(groups < resident ? groups : resident);
+        if constexpr (MODE == kModeDirDot)
+            launch_pdl(k_ax_fx<NX, C, MODE>, grid, fx_threads(NX, C), smem, s, nelt, D, G4, u, w, l2g, eprob, pdone, edot, d);
+        else
+            k_ax_fx<NX, C, MODE><<<grid, fx_threads(NX, C), smem, s>>>(nelt, D, G4, u, w, l2g, eprob, pdone, edot, d);
     } else {
         constexpr size_t smem = ff_smem_bytes<NX, EPB>();
         const int64_t blocks = (nelt + EPB - 1) / EPB;

@@ -34,6 +34,7 @@
 #include "nek_ff.cuh"
 #include "nek_internal.h"
 #include "nek_lines.cuh"
+#include "nek_pdl.cuh"
 #include "nek_reduce.cuh"
 
 namespace nek {
@@ -423,6 +424,7 @@ __global__ void __launch_bounds__(fx_threads(NX, EPB), (fx_min_blocks<NX, EPB>()
     bool dx = false, dp = false;
     double da = 0.0, db = 0.0;
     if constexpr (DIR) {
+        pdl_wait(dir.sc);  // only the matrix has been read so far
         dx = dir.sc->xpend != 0;
         dp = !(dir.sc->done || dir.sc->status != NEK_OK);
         da = dir.sc->alpha;

@@ -38,6 +38,7 @@
 #include <cuda_fp16.h>
 
 #include "nek_internal.h"
+#include "nek_pdl.cuh"
 #include "nek_reduce.cuh"
 #include "nek_tc5.cuh"
 
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(kT5, 4)
     bool dx = false, dp = false;
     float alpha = 0.f, beta = 0.f;
     if constexpr (MODE == kLpDir) {
+        pdl_wait(dir.sc);  // only the matrix has been read so far
         dx = dir.sc->xpend != 0;
         dp = !(dir.sc->done || dir.sc->status != NEK_OK);
         alpha = (float)dir.sc->alpha;
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kT5, 4)
             if (has(k)) {
                 if constexpr (MODE == kLpDir) {
                     in[0][k] = dir.p[o + k * kT5];
-                    in[1][k] = __ldg(dir.r + o + k * kT5);
+                    in[1][k] = dir.r[o + k * kT5];
                     in[2][k] = __ldg(dir.minv + o + k * kT5);
                     in[3][k] = dx ? dir.x[o + k * kT5] : 0.f;
                 } else {
@@ -496,8 +498,11 @@ nek_status launch_tc5_kernel(int64_t nelt, const double* D, const void* Glp, con
     if (!per_sm) per_sm = resident_ctas(reinterpret_cast<const void*>(k_ax_lowp_tc5<S, NX, MODE>), kT5, smem, 8);
     const int64_t cap = (int64_t)per_sm * tc5_sm_count();
     const int grid = static_cast<int>(nelt < cap ? nelt : cap);
-    k_ax_lowp_tc5<S, NX, MODE><<<grid, kT5, smem, s>>>(nelt, D, static_cast<const S*>(Glp), gscale, u, w, edot, dir,
-                                                        kWait5);
+    const S* G = static_cast<const S*>(Glp);
+    if constexpr (MODE == kLpDir)
+        launch_pdl(k_ax_lowp_tc5<S, NX, MODE>, grid, kT5, smem, s, nelt, D, G, gscale, u, w, edot, dir, kWait5);
+    else
+        k_ax_lowp_tc5<S, NX, MODE><<<grid, kT5, smem, s>>>(nelt, D, G, gscale, u, w, edot, dir, kWait5);
     return check_launch();
 }
 

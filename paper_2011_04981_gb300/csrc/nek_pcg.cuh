@@ -39,6 +39,7 @@
 
 #include "nek_ff.cuh"
 #include "nek_internal.h"
+#include "nek_pdl.cuh"
 #include "nek_reduce.cuh"
 
 namespace nek {
@@ -157,17 +158,22 @@ template <class V>
 __global__ void k_dssum_t(int64_t ngroups, const int32_t* __restrict__ off, const int32_t* __restrict__ mem,
                           V* __restrict__ v)
 {
+    pdl_wait();
+    pdl_next();
     dssum_groups<V>(0, ngroups, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, off,
                     mem, v);
 }
 
 template <class V>
-nek_status dssum(const nek_gs* gs, V* v, cudaStream_t s)
+nek_status dssum(const nek_gs* gs, V* v, cudaStream_t s, bool pdl = false)
 {
     if (!gs || gs->ngroups == 0) return NEK_OK;  // no plan: the operator is already assembled
     const int64_t nb = (gs->ngroups + 255) / 256;
-    k_dssum_t<V><<<static_cast<int>(std::min<int64_t>(nb, 152 * 64)), 256, 0, s>>>(gs->ngroups, gs->d_offsets,
-                                                                                 gs->d_members, v);
+    const int blocks = static_cast<int>(std::min<int64_t>(nb, 152 * 64));
+    if (pdl)
+        launch_pdl(k_dssum_t<V>, blocks, 256, 0, s, gs->ngroups, gs->d_offsets, gs->d_members, v);
+    else
+        k_dssum_t<V><<<blocks, 256, 0, s>>>(gs->ngroups, gs->d_offsets, gs->d_members, v);
     return check_launch();
 }
 
@@ -227,6 +233,8 @@ __global__ void __launch_bounds__(NT) k_pw(int64_t n, const V* __restrict__ c, c
                                             const V* __restrict__ p, V* __restrict__ w, double* __restrict__ parts,
                                             const Scalars* __restrict__ sc, const uint8_t* __restrict__ flags)
 {
+    pdl_wait(sc);
+    pdl_next();
     __shared__ double sh[2 * NT];
     if (halted(sc)) return;
     double acc = 0.0;
@@ -272,6 +280,8 @@ __device__ __forceinline__ void set_alpha(double pw, Scalars* sc)
 
 __global__ void __launch_bounds__(NT) k_alpha(const double* __restrict__ parts, int nb, Scalars* sc)
 {
+    pdl_wait(sc);
+    pdl_next();
     __shared__ double sh[NT];
     if (halted(sc)) {
         if (threadIdx.x == 0) sc->xpend = 0;
@@ -287,6 +297,8 @@ constexpr int kAlphaCluster = 8;
 __global__ void __cluster_dims__(kAlphaCluster, 1, 1) __launch_bounds__(NT)
     k_alpha_cluster(const double* __restrict__ parts, int nb, Scalars* sc)
 {
+    pdl_wait(sc);
+    pdl_next();
     __shared__ double sh[NT], mine;
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -333,6 +345,8 @@ __global__ void __launch_bounds__(NT) k_update(int64_t n, const V* __restrict__ 
                                                 const Scalars* __restrict__ sc, const uint8_t* __restrict__ flags,
                                                 const uint8_t* __restrict__ mask)
 {
+    pdl_wait(sc);
+    pdl_next();
     __shared__ double sh[2 * NT];
     if (halted(sc)) return;
     const V alpha = (V)sc->alpha;
@@ -446,6 +460,8 @@ __device__ __forceinline__ void set_beta(double rr, double rz, Scalars* sc)
 
 __global__ void __launch_bounds__(NT) k_beta(const double* __restrict__ parts, int nb, Scalars* sc)
 {
+    pdl_wait(sc);
+    pdl_next();
     __shared__ double sh[2 * NT];
     if (halted(sc)) return;
     double rr, rz;
@@ -459,6 +475,8 @@ template <class V>
 __global__ void k_p(int64_t n, const V* __restrict__ minv, const V* __restrict__ r, V* __restrict__ x,
                     V* __restrict__ p, const Scalars* __restrict__ sc, int update_p)
 {
+    pdl_wait(sc);
+    pdl_next();
     const bool do_x = sc->xpend != 0;
     const bool do_p = update_p && !halted(sc);
     const V alpha = (V)sc->alpha, beta = (V)sc->beta;
@@ -587,19 +605,19 @@ nek_status run(const nek_gs* gs, int64_t n, const V* c, const uint8_t* mask, con
         if (timed) cudaEventRecord(ev[2 * (it - 1)], s);
         if ((st = ax(b.p, b.w, ee ? ee->edot : nullptr, fused ? &dir : nullptr, s)) != NEK_OK) goto done;
         if (timed) cudaEventRecord(ev[2 * (it - 1) + 1], s);
-        if ((st = dssum<V>(gs, b.w, s)) != NEK_OK) goto done;
+        if ((st = dssum<V>(gs, b.w, s, true)) != NEK_OK) goto done;
         if (ee) {
-            k_alpha_cluster<<<kAlphaCluster, NT, 0, s>>>(ee->edot, static_cast<int>(ee->nelt), b.sc);
+            launch_pdl(k_alpha_cluster, kAlphaCluster, NT, 0, s, ee->edot, static_cast<int>(ee->nelt), b.sc);
         } else {
-            k_pw<V><<<nb, NT, 0, s>>>(n, c, mask, b.p, b.w, b.parts, b.sc, flags);
-            k_alpha<<<1, NT, 0, s>>>(b.parts, nb, b.sc);
+            launch_pdl(k_pw<V>, nb, NT, 0, s, n, c, mask, b.p, b.w, b.parts, b.sc, flags);
+            launch_pdl(k_alpha, 1, NT, 0, s, b.parts, nb, b.sc);
             launches += 1;
         }
-        k_update<V><<<nb, NT, 0, s>>>(n, c, minv, b.w, b.r, b.parts, b.sc, flags, mask);
-        k_beta<<<1, NT, 0, s>>>(b.parts, nb, b.sc);
+        launch_pdl(k_update<V>, nb, NT, 0, s, n, c, minv, b.w, b.r, b.parts, b.sc, flags, mask);
+        launch_pdl(k_beta, 1, NT, 0, s, b.parts, nb, b.sc);
         launches += 5;  // the operator, dssum, k_alpha, k_update, k_beta
         if (!fused) {
-            k_p<V><<<sb, 256, 0, s>>>(n, minv, b.r, x, b.p, b.sc, it < max_iter ? 1 : 0);
+            launch_pdl(k_p<V>, sb, 256, 0, s, n, minv, b.r, x, b.p, b.sc, it < max_iter ? 1 : 0);
             launches += 1;
         }
         if ((st = check_launch()) != NEK_OK) goto done;
