@@ -177,7 +177,7 @@ def summarize_clocks(lines):
 
 
 # ------------------------------------------------------------------ helpers
-AX_SOURCES = {"fp64": ("nek_ax.cu", "ax_fp64_traffic.json"), "ff": ("nek_ax_ff_kernels.cuh", "ax_ff_traffic.json"),
+AX_SOURCES = {"fp64": ("nek_ax_dx.cuh", "ax_fp64_traffic.json"), "ff": ("nek_ax_fx.cuh", "ax_ff_traffic.json"),
               "oz": ("nek_ax_oz.cu", "ax_oz_traffic.json")}
 
 

@@ -449,3 +449,25 @@ def test_gradient_batch_sizes_and_alignment(B, shift, with_loss):
         n = int(np.prod(shp))
         _check_elementwise("grad " + name, gg[o:o + n], gr[o:o + n], worst[o:o + n], rms[o:o + n])
         o += n
+
+
+@pytest.mark.parametrize("nelt", [1, 8, 9, 1217])
+def test_prep_conversion_to_single_is_correctly_rounded(nelt):
+    """Elements whose root mean square is a power of two whatever their other values are (two entries of 2^40, the rest
+    below 2^10): every input is then the correctly rounded FP32 value, ties, subnormals and zeros included, bit for bit."""
+    rng = np.random.default_rng(nelt)
+    r = rng.normal(size=(nelt, 512)) * 2.0 ** rng.integers(-130, 4, size=(nelt, 512))
+    ties = rng.integers(1 << 23, 1 << 24, size=(nelt, 100)) * 2.0 + 1.0  # odd: half an ulp of FP32
+    r[:, 100:200] = ties * 2.0 ** rng.integers(-140, -20, size=(nelt, 100))
+    r[:, 200:210] = 0.0
+    r[:, [3, 300]] = 2.0 ** 40
+    r[:, 400:] *= -1.0
+    rd = torch.from_numpy(r).to(DEV)
+    xin = torch.full((nelt, 2, 512), float("nan"), dtype=torch.float32, device=DEV)
+    sc = torch.empty(nelt, dtype=torch.float32, device=DEV)
+    nekax.net_prep(nelt, 8, rd, torch.full_like(rd, 0.5), xin, sc)
+    torch.cuda.synchronize()
+    want = (r * 2.0 ** -36).astype(np.float32)
+    for ch in (0, 1):
+        assert np.array_equal(xin[:, ch].cpu().numpy().view(np.uint32), want.view(np.uint32))
+    assert torch.all(sc == 2.0 ** 35)
