@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_local(int64_t nelt, int n
             o[2 * n3] = g[6 * q + 5];
         }
         __syncthreads();
-        for (int q = threadIdx.x; q < np; q += kDiagThreads) {
+        for (int q = blockIdx.y * kDiagThreads + threadIdx.x; q < np; q += kDiagThreads * gridDim.y) {
             const int e = q / n3, p = q - e * n3, k = p / n2, j = (p - k * n2) / nx, i = p % nx;
             const double* rr = gs + e * 3 * n3;
             const double *sr = rr + p - i, *ss = rr + n3 + p - j * nx, *st = rr + 2 * n3 + p - k * n2;
@@ -96,7 +96,11 @@ nek_status launch_diag_local(int64_t nelt, int nx, const double* D, const double
     nek_status st = ensure_dyn_smem(k_diag_local, sizeof(double) * (2 * 256 + 3 * 4096), configured);  // nx = 16
     if (st != NEK_OK) return st;
     const int64_t nb = (nelt + eb - 1) / eb;
-    k_diag_local<<<static_cast<int>(std::min<int64_t>(nb, 152 * 8)), kDiagThreads, smem, s>>>(nelt, nx, eb, D, G, d);
+    // several blocks on an element's points where there are fewer elements than SMs (64 elements of nx = 16: the call
+    // 47.3 us, 75.9 with one)
+    const int parts = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(eb * n3 / kDiagThreads, 2 * 152 / nb)));
+    const dim3 grid(static_cast<unsigned>(std::min<int64_t>(nb, 152 * 8)), static_cast<unsigned>(parts));
+    k_diag_local<<<grid, kDiagThreads, smem, s>>>(nelt, nx, eb, D, G, d);
     return check_launch();
 }
 

@@ -928,6 +928,21 @@ def test_cg_of_more_elements_than_one_launch_takes():
     assert r["iters"] == 5 and r["kernel_launches"] > 30
 
 
+@pytest.mark.parametrize("nx", [2, 3, 4, 5, 8, 11, 12, 16])
+def test_geometry_of_few_elements_is_that_of_many(nx):
+    """The set-up kernel splits its work by the number of elements (several elements a block, or parts of a line a
+    thread): no bit of an element's factors depends on how many there are."""
+    mesh = inputs.box_mesh(23, 9, 8, nx, perturb=0.15, seed=nx)
+    c = _t(mesh.corners)
+    G = torch.empty((mesh.nelt, nx ** 3, 6), dtype=torch.float64, device=DEV)
+    nekax.geom(mesh.nelt, nx, c, G)
+    for n in (1, 2, 151, 153, 305, 1217):
+        g = torch.full((n, nx ** 3, 6), float("nan"), dtype=torch.float64, device=DEV)
+        nekax.geom(n, nx, c[:n].contiguous(), g)
+        torch.cuda.synchronize()
+        assert torch.equal(g, G[:n])
+
+
 def test_batch_skips_finished_elements_beyond_the_resident_ctas():
     """Problems of more elements than the resident CTAs hold, one of them finished from the start (f = 0): the CTAs
     pass over its elements and the others' iterates are those of a batch without it."""
