@@ -40,7 +40,9 @@ constexpr int BT = 256;       // threads per chunk block
 struct BScal {
     double rz, pw, alpha, beta, rr, bnorm, relres;
     int done, status, iters, it;
-    int xpend;  // this iteration's x += alpha p is still to be applied (kb_p)
+    int xpend;     // this iteration's x += alpha p is still to be applied (kb_p)
+    int rshift;    // r is taken times 2^rshift where its squares are formed in floats; set from bnorm
+    double rback;  // 2^(-2 rshift)
 };
 
 struct Group {
@@ -132,6 +134,8 @@ __global__ void __launch_bounds__(PT) kb_init_finish(const int* __restrict__ pch
         s.rz = rz;
         s.rr = rr;
         s.bnorm = sqrt(rr);
+        s.rshift = pcg::norm_shift(s.bnorm);
+        s.rback = pcg::pow2d(-2 * s.rshift);
         s.relres = 1.0;
         s.status = NEK_OK;
         if (!(rr >= 0.0) || !isfinite(rr) || !isfinite(rz)) {
@@ -210,6 +214,7 @@ __global__ void __launch_bounds__(BT) kb_update(const int64_t* __restrict__ ch_b
     const int64_t a = ch_begin[c], b = ch_begin[c + 1];
     double acc[2] = {0.0, 0.0};
     // <r,r> in float pairs on the FP32 pipes, as the single-problem solve's r update does
+    const int rshift = s.rshift;
     float s_hi = 0.f, s_lo = 0.f, s_c = 0.f;
     for (int64_t q = a + threadIdx.x; q < b; q += BT) {
         const uint8_t fq = flags[q];
@@ -219,11 +224,11 @@ __global__ void __launch_bounds__(BT) kb_update(const int64_t* __restrict__ ch_b
         const double zq = minv[q] * rq;
         r[q] = rq;
         if (fq & pcg::kOwner) {
-            pcg::sq_pair_add(rq, s_hi, s_lo, s_c);
+            pcg::sq_pair_add(rq, rshift, s_hi, s_lo, s_c);
             acc[1] += rq * zq;
         }
     }
-    acc[0] = (widen(s_hi) + widen(s_lo)) + widen(s_c);
+    acc[0] = ((widen(s_hi) + widen(s_lo)) + widen(s_c)) * s.rback;
     chunk_reduce<2>(acc, parts, nchunks, c);
 }
 

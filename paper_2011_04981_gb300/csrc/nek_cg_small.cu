@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(dx_threads(NX, 1, 1), (dx_small_blocks(NX))) k
     const double bt = sc.tol * sc.bnorm, b2 = bt * bt, bh = sc.bnorm * 1e300;
     const double above = sc.tol == 0.0 ? 0.0 : b2 > 1e-280 ? b2 * (1.0 + 1e-13) : INFINITY, huge = fmin(bh * bh, 1e300);
     bool near = true;
+    const int rshift = sc.rshift;
     unsigned target = gridDim.x;
     bool late = !small_barrier(A.bar, target);  // every CTA has read the map: w may be written
     for (int it = 0; it < A.max_iter && !late && !halted(&sc); it++) {
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(dx_threads(NX, 1, 1), (dx_small_blocks(NX))) k
                 const unsigned f = fl >> (2 * b);
                 r[b] = fma(-alpha, f & kFree ? w[b] : 0.0, r[b]);
                 if (f & kOwner) {
-                    sq_pair_add(r[b], s_hi, s_lo, s_c);
+                    sq_pair_add(r[b], rshift, s_hi, s_lo, s_c);
                     v2[1] += r[b] * (mi[b] * r[b]);
                 }
             }
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(dx_threads(NX, 1, 1), (dx_small_blocks(NX))) k
         if ((late = !small_wait(A.bar, target += gridDim.x))) break;
         // the residual test and beta, the same operations as set_beta, one warp each
         if (tid < 32) {
-            const double rr = small_sum(A.parts, A.nelt);
+            const double rr = small_sum(A.parts, A.nelt) * sc.rback;
             if (tid == 0) {
                 sc.rr = rr;
                 near = !(rr > above && rr <= huge);

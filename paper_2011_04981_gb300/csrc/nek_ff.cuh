@@ -28,6 +28,19 @@ __device__ __forceinline__ float2 split_double(double x)
     return make_float2(h, e >= 943 ? __uint_as_float(__float_as_uint(l) | sgn) : 0.0f);
 }
 
+// The same of x 2^k, for |k| <= 500 and every x: magnitudes below 2^-126 give zero or a subnormal, from 2^128 on
+// (and infinities, NaNs) a value that is not finite.
+__device__ __forceinline__ float2 split_double_shift(double x, int k)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned sgn = hi & 0x80000000u;
+    const int e = max(896, min(1151, (int)((hi >> 20) & 0x7FFu) + k));
+    const float h = __uint_as_float(sgn | ((unsigned)(e - 896) << 23) | (((hi & 0xFFFFFu) << 3) | (lo >> 29)));
+    const float r = __fsub_rn(__uint_as_float(0x4B000000u | ((lo >> 6) & 0x7FFFFFu)), 8388608.0f);
+    const float l = __fmul_rn(r, __uint_as_float(sgn | ((unsigned)(e - 942) << 23)));
+    return make_float2(h, e >= 943 ? l : 0.0f);
+}
+
 // (double)h + (double)l with the two widenings done by integer operations and a
 // single FP64 add.
 __device__ __forceinline__ double widen(float f)

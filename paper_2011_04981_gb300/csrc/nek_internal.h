@@ -111,6 +111,8 @@ struct PcgScalars {
     int iters;      // iterations completed when done/status was set
     int it;         // iterations executed so far
     int xpend;      // this iteration's x += alpha p is still to be applied
+    int rshift;     // r is taken times 2^rshift where its squares are formed in floats; set from bnorm
+    double rback;   // 2^(-2 rshift)
 };
 
 // The PCG direction update done by the float-float operator as it loads its

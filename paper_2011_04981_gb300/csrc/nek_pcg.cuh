@@ -105,6 +105,15 @@ __device__ __forceinline__ bool is_free(const uint8_t* __restrict__ mask, const 
     return flags ? (flags[q] & kFree) != 0 : mask[q] != 0;
 }
 
+// The shift that brings values of the size of bnorm near one, within what k_update's sums can take back.
+__device__ __forceinline__ int norm_shift(double bnorm)
+{
+    const int e = ((__double2hiint(bnorm) >> 20) & 0x7FF) - 1023;  // bnorm = 0: the shift is not used
+    return max(-500, min(500, -e));
+}
+// 2^e, -1022 <= e <= 1023.
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+
 inline size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 inline int stream_blocks(int64_t n)
@@ -209,6 +218,8 @@ __global__ void __launch_bounds__(NT) k_init_finish(const double* __restrict__ p
         sc->rz = rz;
         sc->rr = rr;
         sc->bnorm = sqrt(rr);
+        sc->rshift = norm_shift(sc->bnorm);
+        sc->rback = pow2d(-2 * sc->rshift);
         sc->tol = tol;
         sc->it = 0;
         sc->iters = 0;
@@ -323,13 +334,14 @@ __global__ void __cluster_dims__(kAlphaCluster, 1, 1) __launch_bounds__(NT)
     cluster.sync();  // the blocks' sums stay until they are read
 }
 
-// r -= alpha mask.w; partials of <r,r>_c and <r,z>_c with z = minv r (not stored)
-// (s_hi + s_lo) + s_c += r^2 in float pairs: r = rh + rl split by integer operations (|r - rh - rl| <=
-// 2^-46 |r|), r^2 = rh^2 (exact as the float pair p + e) + 2 rh rl; p summed with TwoSum into s_hi + s_lo,
-// e + 2 rh rl into s_c.  For sums of ~100 terms a thread: good to ~2^-40 of the sum.
-__device__ __forceinline__ void sq_pair_add(double r, float& s_hi, float& s_lo, float& s_c)
+// (s_hi + s_lo) + s_c += (r 2^k)^2 in float pairs: r 2^k = rh + rl split by integer operations (to 2^-46 of it), its
+// square = rh^2 (exact as the float pair p + e) + 2 rh rl; p summed with TwoSum into s_hi + s_lo, e + 2 rh rl into s_c.
+// For sums of ~100 terms a thread: good to ~2^-40 of the sum.  With k = norm_shift(bnorm) the squares stay in the range
+// of floats whatever the size of the right-hand side is: up to 2^63 times bnorm (beyond it the sum is not finite), and
+// down to 2^-63 of it (smaller values count as zero).
+__device__ __forceinline__ void sq_pair_add(double r, int k, float& s_hi, float& s_lo, float& s_c)
 {
-    const float2 h = split_double(r);
+    const float2 h = split_double_shift(r, k);
     const float pr = __fmul_rn(h.x, h.x);
     const float t = __fmaf_rn(2.f * h.x, h.y, __fmaf_rn(h.x, h.x, -pr));
     const float sn = __fadd_rn(s_hi, pr);
@@ -339,6 +351,7 @@ __device__ __forceinline__ void sq_pair_add(double r, float& s_hi, float& s_lo, 
     s_c = __fadd_rn(s_c, t);
 }
 
+// r -= alpha mask.w; partials of <r,r>_c and <r,z>_c with z = minv r (not stored)
 template <class V>
 __global__ void __launch_bounds__(NT) k_update(int64_t n, const V* __restrict__ c, const V* __restrict__ minv,
                                                 const V* __restrict__ w, V* __restrict__ r, double* __restrict__ parts,
@@ -405,7 +418,8 @@ __global__ void __launch_bounds__(NT) k_update(int64_t n, const V* __restrict__ 
         // the FP32 pipes, so that GB300's 2-per-clock FP64 pipe carries three operations a point, not four:
         // r = rh + rl split by integer operations (|r - rh - rl| <= 2^-46 |r|), r^2 = rh^2 (exact as the
         // float pair p + e) + 2 rh rl, the p summed with TwoSum, the rest in plain floats: each thread's sum
-        // is good to ~2^-40 of itself
+        // is good to ~2^-40 of itself.  r is taken times a power of two (rshift), so the floats' range does not show
+        const int rshift = sc->rshift;
         float s_hi = 0.f, s_lo = 0.f, s_c = 0.f;
 #pragma unroll 4
         for (int64_t q = blockIdx.x * (int64_t)NT + threadIdx.x; q < n; q += stride) {
@@ -418,14 +432,14 @@ __global__ void __launch_bounds__(NT) k_update(int64_t n, const V* __restrict__ 
             if (fq & kOwner) {
                 arz += to_f64(rq) * to_f64(zq);
                 if constexpr (std::is_same<V, double>::value) {
-                    sq_pair_add(rq, s_hi, s_lo, s_c);
+                    sq_pair_add(rq, rshift, s_hi, s_lo, s_c);
                 } else {
                     const double rd = to_f64(rq);
                     arr += rd * rd;
                 }
             }
         }
-        if constexpr (std::is_same<V, double>::value) arr = (widen(s_hi) + widen(s_lo)) + widen(s_c);
+        if constexpr (std::is_same<V, double>::value) arr = ((widen(s_hi) + widen(s_lo)) + widen(s_c)) * sc->rback;
     } else {
         for (int64_t q = blockIdx.x * (int64_t)NT + threadIdx.x; q < n; q += stride) {
             V wv = w[q];

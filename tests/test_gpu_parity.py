@@ -963,3 +963,45 @@ def test_batch_skips_finished_elements_beyond_the_resident_ctas():
     assert torch.all(xs[1] == 0)
     for a, b in ((xs[0], ys[0]), (xs[2], ys[1])):
         assert torch.all(torch.isfinite(b)) and float((a - b).abs().max()) <= 1e-9 * float(b.abs().max())
+
+
+# ------------------------------------------------- scale of the right-hand side
+@pytest.mark.parametrize("path,e", [("one launch", -90), ("one launch", 90), ("loop", -90), ("loop", 90), ("loop", 0),
+                                    ("float-float", 70), ("one launch", -450), ("loop", 450)])
+def test_cg_of_a_scaled_right_hand_side(path, e):
+    """2^e f: every operation of the solve scales exactly, so the iteration count, the residual and, but for the power of
+    two, every bit of x are those of f, also where the squares of r leave the range of FP32.  Beyond 2^+-400 the FP64
+    operator sums its lines in FP64, in another order: there the oracle's residual is compared."""
+    mesh = inputs.box_mesh(4, 3, 3, 6, perturb=0.1, seed=2)
+    P = DeviceProblem(mesh, DEV)
+    fh = inputs.random_global_field(mesh, seed=3)
+    f = _t(fh)
+    g = f * 2.0 ** e
+    kw = dict(tol=1e-9, max_iter=1000, time_ax=path == "loop", ax_impl=nekax.AX_FF if path == "float-float" else nekax.AX_FP64)
+    x, y = torch.empty_like(f), torch.empty_like(f)
+    a, b = P.cg(f, x, **kw), P.cg(g, y, **kw)
+    assert a["status"] == b["status"] == nekax.OK and a["iters"] > 20
+    if abs(e) < 400:
+        assert (a["iters"], a["relres"]) == (b["iters"], b["relres"])
+        assert torch.equal(y, x * 2.0 ** e)
+    else:
+        yh = (y * 2.0 ** -e).cpu().numpy().reshape(mesh.nelt, -1)
+        assert ref.Problem(mesh).residual(fh, yh) <= 1e-9 * 1.001
+
+
+@pytest.mark.parametrize("per_graph", [10, -1])
+def test_batch_of_scaled_right_hand_sides(per_graph):
+    """The same problem four times in a batch, with f of the sizes 1, 2^-90, 2^90 and 2^-300."""
+    from paper_2011_04981_gb300.problem import DeviceBatch
+
+    mesh = inputs.box_mesh(4, 3, 3, 6, perturb=0.1, seed=2)
+    fh = inputs.random_global_field(mesh, seed=3)
+    ex = [0, -90, 90, -300]
+    B = DeviceBatch([mesh] * 4, [np.ldexp(fh, e) for e in ex], DEV, ff=False)
+    x = torch.full((B.npts,), float("nan"), dtype=torch.float64, device=DEV)
+    r = B.solve(x, tol=1e-9, max_iter=1000, iters_per_graph=per_graph)
+    assert r["status"] == nekax.OK and r["iters"][0] > 20
+    assert np.all(r["iters"] == r["iters"][0]) and np.all(r["relres"] == r["relres"][0])
+    xs = [v.cpu().numpy() for v in B.split(x)]
+    for v, e in zip(xs, ex):
+        assert np.array_equal(v, np.ldexp(xs[0], e))
