@@ -574,6 +574,15 @@ nek_status nek_cg_solve_ex(const nek_gs* gs, int64_t nelt, int nx, const double*
                            int max_iter, void* workspace, int* iters_out, double* relres_out, nek_cg_opts* opts,
                            void* stream);
 
+/* Self-test of the bounded waits of the FP64 solve of few elements: nek_cg_solve with every wait of its one-launch form
+ * bounded by wait_us microseconds (1 .. 2e6; 2e6 in the solve itself).  force_timeout != 0: no wait is ever met, so the
+ * kernel must give up and return, and the loop of launches solves in its place; the result is the loop's, and
+ * *kernel_launches (not null) counts both.  For tests. */
+nek_status nek_cg_selftest(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G,
+                           const uint8_t* mask, const double* minv, const double* f, double* x, double tol_rel,
+                           int max_iter, int force_timeout, int64_t wait_us, int* iters_out, double* relres_out,
+                           int* kernel_launches, void* stream);
+
 /* Same solve with f and x in HOST memory (pinned or pageable), for callers
  * whose right-hand side and solution live on the host: f_host is copied to the
  * device, the solve of nek_cg_solve_ex runs, and x is copied back to x_host;

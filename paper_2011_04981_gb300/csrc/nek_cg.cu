@@ -159,10 +159,12 @@ size_t nek_cg_workspace_bytes(int64_t nelt, int nx, int need_minv)
            pcg::align256(sizeof(double) * 2 * kMaxReduceBlocks) + pcg::align256(sizeof(pcg::Scalars));
 }
 
-nek_status nek_cg_solve_ex(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G,
+}  // extern "C"
+
+static nek_status cg_solve(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G,
                            const uint8_t* mask, const double* minv, const double* f, double* x, double tol_rel,
                            int max_iter, void* workspace, int* iters_out, double* relres_out, nek_cg_opts* opts,
-                           void* stream)
+                           void* stream, const pcg::SmallWait& wait)
 {
     if (iters_out) *iters_out = 0;
     if (relres_out) *relres_out = 0.0;
@@ -238,11 +240,15 @@ nek_status nek_cg_solve_ex(const nek_gs* gs, int64_t nelt, int nx, const double*
                                           : launch_ax_fp64(nelt, nx, D, G, p, w, ss);
         };
         bool ran = false;
+        const double* rhs = f;
         if (ax_impl == NEK_AX_FP64 && !time_ax)
-            st = pcg::run_small(gs, nelt, nx, D, G, mask, mv, flags, f, x, b, edot, tol_rel, max_iter, s, &res, ran);
-        if (!ran && st == NEK_OK)
-            st = pcg::run<double>(gs, n, gs->d_c, mask, mv, f, x, b, tol_rel, max_iter, check_every, time_ax, ax, s,
+            st = pcg::run_small(gs, nelt, nx, D, G, mask, mv, flags, f, x, b, edot, tol_rel, max_iter, s, &res, ran, rhs,
+                                wait);
+        if (!ran && st == NEK_OK) {
+            extra += res.launches;
+            st = pcg::run<double>(gs, n, gs->d_c, mask, mv, rhs, x, b, tol_rel, max_iter, check_every, time_ax, ax, s,
                                   &res, flags, energies ? &ee : nullptr);
+        }
         if (iters_out) *iters_out = res.iters;
         if (relres_out) *relres_out = res.relres;
         if (opts) {
@@ -256,6 +262,30 @@ nek_status nek_cg_solve_ex(const nek_gs* gs, int64_t nelt, int nx, const double*
         nek_status st2 = check_cuda(cudaStreamSynchronize(s));
         if (st == NEK_OK) st = st2;
     }
+    return st;
+}
+
+extern "C" {
+
+nek_status nek_cg_solve_ex(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G,
+                           const uint8_t* mask, const double* minv, const double* f, double* x, double tol_rel,
+                           int max_iter, void* workspace, int* iters_out, double* relres_out, nek_cg_opts* opts,
+                           void* stream)
+{
+    return cg_solve(gs, nelt, nx, D, G, mask, minv, f, x, tol_rel, max_iter, workspace, iters_out, relres_out, opts, stream,
+                    pcg::SmallWait{});
+}
+
+nek_status nek_cg_selftest(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G,
+                           const uint8_t* mask, const double* minv, const double* f, double* x, double tol_rel,
+                           int max_iter, int force_timeout, int64_t wait_us, int* iters_out, double* relres_out,
+                           int* kernel_launches, void* stream)
+{
+    if (wait_us < 1 || wait_us > 2000000 || !kernel_launches) return NEK_ERR_INVALID_ARG;
+    nek_cg_opts opts{};
+    const nek_status st = cg_solve(gs, nelt, nx, D, G, mask, minv, f, x, tol_rel, max_iter, nullptr, iters_out, relres_out,
+                                   &opts, stream, pcg::SmallWait{wait_us * 1000ll, force_timeout != 0});
+    *kernel_launches = opts.kernel_launches;
     return st;
 }
 

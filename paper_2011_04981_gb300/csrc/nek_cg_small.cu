@@ -32,13 +32,10 @@ struct SmallArgs {
     Scalars* sc;
     unsigned* bar;  // arrivals, zero at the start
     int max_iter;
+    long long wait_ns;
 };
 
-// A wait that is not met within this many polls (some seconds; the launch is cooperative, so every CTA is resident and it
-// is met) ends the kernel, and the general loop solves instead.
-constexpr int kSpinLimit = 1 << 22;
-
-// Iterations of one launch at most: keeps it below half a second or so.
+// Iterations of one launch at most: about a second (1.1 s at nx = 16).
 constexpr int kSmallMaxIter = 20000;
 
 namespace {
@@ -51,31 +48,48 @@ constexpr int dx_small_blocks(int nx)
     return b < 1 ? 1 : b;
 }
 
-// The barrier of all CTAs, in two halves; the wait is false if it ran out.
+__device__ __forceinline__ long long now_ns()
+{
+    long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// The barrier of all CTAs, in two halves.  The launch is cooperative, so every CTA is resident and the wait is met; one
+// that is not within wait_ns is false, which ends the kernel, and the general loop solves instead.
 __device__ __forceinline__ void small_arrive(unsigned* bar)
 {
     __syncthreads();
     if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
 }
 
-__device__ __forceinline__ bool small_wait(unsigned* bar, unsigned target)
+__device__ __forceinline__ bool small_wait(unsigned* bar, unsigned target, long long wait_ns)
 {
     bool late = false;
     if (threadIdx.x == 0) {
-        unsigned v;
-        int n = 0;
-        do {
+        long long t0 = 0;
+        for (unsigned n = 1;; n++) {
+            unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-        } while ((int)(v - target) < 0 && ++n < kSpinLimit);
-        late = (int)(v - target) < 0;
+            if ((int)(v - target) >= 0) break;
+            if ((n & 63u) == 0u) {  // the clock is looked at from the 64th poll on (some 50 us)
+                const long long t = now_ns();
+                if (t0 == 0)
+                    t0 = t;
+                else if (t - t0 > wait_ns) {
+                    late = true;
+                    break;
+                }
+            }
+        }
     }
     return !__syncthreads_or(late);
 }
 
-__device__ __forceinline__ bool small_barrier(unsigned* bar, unsigned target)
+__device__ __forceinline__ bool small_barrier(unsigned* bar, unsigned target, long long wait_ns)
 {
     small_arrive(bar);
-    return small_wait(bar, target);
+    return small_wait(bar, target, wait_ns);
 }
 
 // Sum of n values by one warp, in a fixed order, in every lane; past the L1 (other CTAs wrote them).
@@ -150,7 +164,7 @@ __global__ void __launch_bounds__(dx_threads(NX, 1, 1), (dx_small_blocks(NX))) k
     bool near = true;
     const int rshift = sc.rshift;
     unsigned target = gridDim.x;
-    bool late = !small_barrier(A.bar, target);  // every CTA has read the map: w may be written
+    bool late = !small_barrier(A.bar, target, A.wait_ns);  // every CTA has read the map: w may be written
     for (int it = 0; it < A.max_iter && !late && !halted(&sc); it++) {
         // ---- w = A_e p
         if (active) dx_lines<NX, false, 1>(ln.u, ln.a, ln.str, ln.sgn, S.tab[0], S.D, sym, bad);
@@ -168,7 +182,7 @@ __global__ void __launch_bounds__(dx_threads(NX, 1, 1), (dx_small_blocks(NX))) k
                 if (gn[b]) A.w[e0 + t + b * TPE] = w[b];
             }
         }
-        if ((late = !small_barrier(A.bar, target += gridDim.x))) break;
+        if ((late = !small_barrier(A.bar, target += gridDim.x, A.wait_ns))) break;
         // ---- dssum of the own points, <p,w>
         double pw[1] = {0.0}, o1[B];
 #pragma unroll
@@ -196,7 +210,7 @@ __global__ void __launch_bounds__(dx_threads(NX, 1, 1), (dx_small_blocks(NX))) k
             const double v = block_sums<NB, 1>(pw, sh);
             if (tid == 0) A.pwparts[blockIdx.x] = v;
         }
-        if ((late = !small_barrier(A.bar, target += gridDim.x))) break;
+        if ((late = !small_barrier(A.bar, target += gridDim.x, A.wait_ns))) break;
         if (tid < 32) {
             const double s = small_sum(A.pwparts, A.nelt);
             if (tid == 0) set_alpha(s, &sc);
@@ -227,7 +241,7 @@ __global__ void __launch_bounds__(dx_threads(NX, 1, 1), (dx_small_blocks(NX))) k
 #pragma unroll
         for (int b = 0; b < B; b++)
             if (has(b)) x[b] = fma(alpha, Ut[off(b)], x[b]);
-        if ((late = !small_wait(A.bar, target += gridDim.x))) break;
+        if ((late = !small_wait(A.bar, target += gridDim.x, A.wait_ns))) break;
         // the residual test and beta, the same operations as set_beta, one warp each
         if (tid < 32) {
             const double rr = small_sum(A.parts, A.nelt) * sc.rback;
@@ -298,7 +312,8 @@ nek_status launch_small(const SmallArgs& a, cudaStream_t s, bool& ran)
 
 nek_status run_small(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G, const uint8_t* mask,
                      const double* minv, const uint8_t* flags, const double* f, double* x, const Buffers<double>& b,
-                     double* edot, double tol, int max_iter, cudaStream_t s, Result* res, bool& ran)
+                     double* edot, double tol, int max_iter, cudaStream_t s, Result* res, bool& ran, const double*& rhs,
+                     const SmallWait& wait)
 {
     ran = false;
     if (nx < 4 || nelt > (int64_t)kSMs * dx_small_blocks(nx) || nelt > kMaxReduceBlocks || max_iter > kSmallMaxIter)
@@ -321,10 +336,13 @@ nek_status run_small(const nek_gs* gs, int64_t nelt, int nx, const double* D, co
     a.sc = b.sc;
     a.bar = reinterpret_cast<unsigned*>(b.sc + 1);
     a.max_iter = max_iter;
+    a.wait_ns = wait.ns;
     k_init<double><<<nb, NT, 0, s>>>(n, gs->d_c, mask, minv, f, x, b.r, b.p, b.parts, flags);
     k_init_finish<<<1, NT, 0, s>>>(b.parts, nb, tol, b.sc);
+    rhs = b.r;  // masked f, which the kernel leaves as it is; f itself may lie where x is
     int launches = 2;
-    nek_status st = check_cuda(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s));
+    // (for the self-test: the counter one short, so that no wait is met)
+    nek_status st = check_cuda(cudaMemsetAsync(a.bar, wait.force_timeout ? 0xFF : 0, sizeof(unsigned), s));
     if (st != NEK_OK) return st;
     if (gs->ngroups > 0) {
         if ((st = check_cuda(cudaMemsetAsync(b.w, 0xFF, sizeof(int32_t) * n, s))) != NEK_OK) return st;
@@ -352,6 +370,7 @@ nek_status run_small(const nek_gs* gs, int64_t nelt, int nx, const double* D, co
         case 16: st = launch_small<16>(a, s, ran); break;
         default: return NEK_OK;
     }
+    res->launches = launches + (ran ? 1 : 0);
     if (st != NEK_OK || !ran) return st;
     Scalars h{};
     if ((st = check_cuda(cudaMemcpyAsync(&h, b.sc, sizeof(h), cudaMemcpyDeviceToHost, s))) != NEK_OK) return st;
@@ -360,7 +379,6 @@ nek_status run_small(const nek_gs* gs, int64_t nelt, int nx, const double* D, co
         ran = false;
         return NEK_OK;
     }
-    res->launches = launches + 1;
     return result_of(h, tol, res);
 }
 

@@ -578,13 +578,22 @@ inline nek_status result_of(const Scalars& h, double tol, Result* res)
     return tol > 0.0 && !h.done ? NEK_ERR_NOT_CONVERGED : NEK_OK;
 }
 
-// The FP64 solve of few elements in one launch (nek_cg_small.cu): ran is false, and nothing but the buffers written,
-// where the elements or the iterations are too many for it.  edot: nelt doubles of scratch; the rest as run.
+// The bound of the one-launch solve's waits; force_timeout (for the self-test): none of them is met.
+struct SmallWait {
+    long long ns = 2000000000ll;
+    bool force_timeout = false;
+};
+
+// The FP64 solve of few elements in one launch (nek_cg_small.cu).  ran is false where the elements or the iterations are
+// too many for it, or where one of its waits ran out: the caller then solves from rhs, which is f, or the masked f in
+// b.r once x has been written; res->launches are the kernels it enqueued all the same.  edot: nelt doubles of scratch; the
+// rest as run.
 nek_status run_small(const nek_gs* gs, int64_t nelt, int nx, const double* D, const double* G, const uint8_t* mask,
                      const double* minv, const uint8_t* flags, const double* f, double* x, const Buffers<double>& b,
-                     double* edot, double tol, int max_iter, cudaStream_t s, Result* res, bool& ran);
+                     double* edot, double tol, int max_iter, cudaStream_t s, Result* res, bool& ran, const double*& rhs,
+                     const SmallWait& wait);
 
-// Runs PCG from x = 0.  `ax(p, w, edot, dir, stream)` applies the element
+// Runs PCG from x = 0; f may be b.r or x.  `ax(p, w, edot, dir, stream)` applies the element
 // operator, which gs then sums over shared nodes; with gs null, ax applies the
 // assembled operator itself.  edot is ee->edot on the element-energy path (ee
 // non-null), else null; dir is the direction update the operator applies

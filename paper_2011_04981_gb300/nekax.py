@@ -143,6 +143,7 @@ _SIGS = {
     "nek_cg_solve": ([_P, _I64, _I, _P, _P, _P, _P, _P, _P, _D, _I, _P, _P, _P, _P], _I),
     "nek_cg_solve_ex": ([_P, _I64, _I, _P, _P, _P, _P, _P, _P, _D, _I, _P, _P, _P, ctypes.POINTER(NekCgOpts), _P],
                         _I),
+    "nek_cg_selftest": ([_P, _I64, _I, _P, _P, _P, _P, _P, _P, _D, _I, _I, _I64, _P, _P, _P, _P], _I),
     "nek_cg_host_staging_bytes": ([_I64, _I], ctypes.c_size_t),
     "nek_cg_solve_host": ([_P, _I64, _I, _P, _P, _P, _P, _P, _P, _D, _I, _P, _P, _P, _P, ctypes.POINTER(NekCgOpts),
                            _P], _I),
@@ -530,6 +531,18 @@ def cg_solve(gs: GsPlan, nelt, nx, D, G, m, minv, f, x, tol=1e-8, max_iter=1000,
         raise NekError("nek_cg_solve", st)
     return dict(status=st, iters=it.value, relres=rr.value, ax_ms_total=opts.ax_ms_total,
                 ax_launches=opts.ax_launches, kernel_launches=opts.kernel_launches)
+
+
+def cg_selftest(gs: GsPlan, nelt, nx, D, G, m, minv, f, x, tol=1e-8, max_iter=1000, force_timeout=True, wait_us=20000,
+                stream=None):
+    """Self-test of the one-launch solve's bounded waits (nek_cg_selftest); returns dict(status, iters, relres, kernel_launches)."""
+    it, rr, kl = _I(0), _D(0.0), _I(0)
+    st = load().nek_cg_selftest(gs.handle, nelt, nx, _ptr(D), _ptr(G), _ptr(m), _ptr(minv), _ptr(f), _ptr(x), float(tol),
+                                int(max_iter), 1 if force_timeout else 0, int(wait_us), ctypes.byref(it),
+                                ctypes.byref(rr), ctypes.byref(kl), _stream(stream))
+    if st not in (OK, ERR_NOT_CONVERGED, ERR_BREAKDOWN):
+        raise NekError("nek_cg_selftest", st)
+    return dict(status=st, iters=it.value, relres=rr.value, kernel_launches=kl.value)
 
 
 def cg_host_staging_bytes(nelt, nx):

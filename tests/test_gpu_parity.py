@@ -1005,3 +1005,33 @@ def test_batch_of_scaled_right_hand_sides(per_graph):
     xs = [v.cpu().numpy() for v in B.split(x)]
     for v, e in zip(xs, ex):
         assert np.array_equal(v, np.ldexp(xs[0], e))
+
+
+# ------------------------------------------------- bounded waits of the one-launch solve
+@pytest.mark.parametrize("dims,nx", [((4, 3, 3), 6), ((8, 19, 1), 12)])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_one_launch_solve_whose_waits_run_out(dims, nx, in_place):
+    """No wait of the one-launch solve is met: its kernel gives up within the bound, and the loop of launches solves in
+    its place: the loop's result to the bit, also where x takes the place of f, with the given-up kernels counted.  The
+    context stays usable and the one-launch solve then runs as ever."""
+    import time
+
+    mesh = inputs.box_mesh(*dims, nx, perturb=0.1, seed=nx)
+    P = DeviceProblem(mesh, DEV)
+    f = _t(inputs.random_global_field(mesh, seed=3))
+    x, y = torch.empty_like(f), torch.empty_like(f)
+    loop = P.cg(f, x, tol=1e-7, max_iter=2000, time_ax=True)
+    fast = P.cg(f, y, tol=1e-7, max_iter=2000)
+    assert fast["kernel_launches"] <= 10 < loop["kernel_launches"]
+    z = f.clone() if in_place else torch.full_like(f, 3.0)
+    args = (P.gs, mesh.nelt, nx, P.D, P.G, P.mask, P.minv, z if in_place else f, z, 1e-7, 2000)
+    torch.cuda.synchronize()
+    t = time.perf_counter()
+    r = nekax.cg_selftest(*args, force_timeout=True, wait_us=20000)
+    assert time.perf_counter() - t < 1.5
+    assert (r["status"], r["iters"], r["relres"]) == (loop["status"], loop["iters"], loop["relres"])
+    assert torch.equal(z, x) and r["kernel_launches"] > loop["kernel_launches"]
+    if in_place:
+        z.copy_(f)
+    r = nekax.cg_selftest(*args, force_timeout=False, wait_us=2000000)
+    assert r["kernel_launches"] == fast["kernel_launches"] and r["iters"] == fast["iters"] and torch.equal(z, y)
