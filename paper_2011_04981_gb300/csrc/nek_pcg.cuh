@@ -291,7 +291,7 @@ __device__ __forceinline__ void set_alpha(double pw, Scalars* sc)
 
 __global__ void __launch_bounds__(NT) k_alpha(const double* __restrict__ parts, int nb, Scalars* sc)
 {
-    pdl_wait(sc);
+    pdl_wait(sc, parts);
     pdl_next();
     __shared__ double sh[NT];
     if (halted(sc)) {
@@ -308,7 +308,7 @@ constexpr int kAlphaCluster = 8;
 __global__ void __cluster_dims__(kAlphaCluster, 1, 1) __launch_bounds__(NT)
     k_alpha_cluster(const double* __restrict__ parts, int nb, Scalars* sc)
 {
-    pdl_wait(sc);
+    pdl_wait(sc, parts);
     pdl_next();
     __shared__ double sh[NT], mine;
     namespace cg = cooperative_groups;
@@ -474,7 +474,7 @@ __device__ __forceinline__ void set_beta(double rr, double rz, Scalars* sc)
 
 __global__ void __launch_bounds__(NT) k_beta(const double* __restrict__ parts, int nb, Scalars* sc)
 {
-    pdl_wait(sc);
+    pdl_wait(sc, parts);
     pdl_next();
     __shared__ double sh[2 * NT];
     if (halted(sc)) return;

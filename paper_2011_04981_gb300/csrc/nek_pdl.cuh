@@ -16,9 +16,12 @@
 namespace nek {
 
 // p...: pointers that the wait redefines, so that no load through them, const __restrict__ or not, can be moved above
-// it.  The kernels give their scalars: what else they read comes after a test of these, or through pointers that are written
-// in the same kernel or by instructions that stay in order.  (Redefining all of k_ax_fx's DirUpdate takes it from the constant
-// bank into registers: 10.25 -> 10.57 ms for the 20 iterations.)
+// it, or be made a read-only one.  A kernel gives its scalars, and what else the kernel just before it may still write
+// while this one runs, where it is a const __restrict__ parameter (which may be read as data that nothing writes for as
+// long as the kernel runs): k_alpha's and k_beta's partial sums.  What lies further back is complete before this kernel
+// starts; it is read after a test of the scalars, or through pointers that are written in the same kernel.
+// (Redefining all of k_ax_fx's DirUpdate takes it from the constant bank into registers: 10.25 -> 10.57 ms for the 20
+// iterations.)
 template <class... P>
 __device__ __forceinline__ void pdl_wait(P&... p)
 {
