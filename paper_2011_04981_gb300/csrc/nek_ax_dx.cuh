@@ -396,12 +396,21 @@ __global__ void __launch_bounds__(dx_threads(NX, EPB, LPT), (dx_min_blocks<NX, E
 constexpr int dx_conc(int nx, int epb) { return nx >= 9 ? 1 : epb; }
 
 template <int NX, int EPB, int LPT>
-nek_status launch_dx_kernel(int64_t nelt, const double* D, const double* G, const double* u, double* w, cudaStream_t s)
+nek_status configure_dx()
 {
     constexpr size_t smem = sizeof(DxSmem<NX, EPB>);
     static_assert(smem <= 227 * 1024 && dx_threads(NX, EPB, LPT) <= 1024, "fits an SM");
     static std::atomic<uint64_t> configured{0};
-    nek_status st = ensure_dyn_smem(k_ax_dx<NX, EPB, LPT>, smem, configured);
+    return ensure_dyn_smem(k_ax_dx<NX, EPB, LPT>, smem, configured);
+}
+
+template <int NX, int EPB, int LPT>
+nek_status launch_dx_kernel(int64_t nelt, const double* D, const double* G, const double* u, double* w, cudaStream_t s)
+{
+    constexpr size_t smem = sizeof(DxSmem<NX, EPB>);
+    nek_status st = configure_dx<NX, EPB, LPT>();
+    // and the form of few elements: a solve whose launches shrink to it may first do so inside a graph's capture
+    if (st == NEK_OK) st = configure_dx<NX, 1, 1>();
     if (st != NEK_OK) return st;
     const int64_t groups = (nelt + EPB - 1) / EPB, resident = kSMs * dx_min_blocks<NX, EPB, LPT>();
     k_ax_dx<NX, EPB, LPT><<<(unsigned)(groups < resident ? groups : resident), dx_threads(NX, EPB, LPT), smem, s>>>(

@@ -1035,3 +1035,35 @@ def test_one_launch_solve_whose_waits_run_out(dims, nx, in_place):
         z.copy_(f)
     r = nekax.cg_selftest(*args, force_timeout=False, wait_us=2000000)
     assert r["kernel_launches"] == fast["kernel_launches"] and r["iters"] == fast["iters"] and torch.equal(z, y)
+
+
+_SHRINKING_BATCH = """
+import sys
+sys.path.insert(0, %r)
+import numpy as np, torch
+from paper_2011_04981_gb300 import inputs, nekax
+from paper_2011_04981_gb300.problem import DeviceBatch
+nx = %d
+meshes = [inputs.box_mesh(10, 5, 2, nx, perturb=0.1, seed=1), inputs.box_mesh(12, 5, 2, nx, perturb=0.1, seed=2)]
+f = [np.zeros((100, nx ** 3)), inputs.random_global_field(meshes[1], seed=3)]
+B = DeviceBatch(meshes, f, "cuda", ff=False)
+x = torch.full((B.npts,), float("nan"), dtype=torch.float64, device="cuda")
+r = B.solve(x, tol=1e-7, max_iter=500, iters_per_graph=10)
+y = torch.full_like(x, float("nan"))
+e = B.solve(y, tol=1e-7, max_iter=500, iters_per_graph=0)
+assert r["status"] == e["status"] == nekax.OK and r["graph_launches"] > 1 and e["graph_launches"] == 0
+assert np.array_equal(r["iters"], e["iters"]) and min(r["iters"]) == 0 and torch.equal(x, y)
+"""
+
+
+@pytest.mark.parametrize("nx", [4, 8, 11])
+def test_batch_whose_fp64_launches_shrink_inside_captures(nx):
+    """220 elements of one order, 100 of them finished from the start: the operator's launch falls to 120 elements, where
+    it takes its form of few elements, for the first time in the process in a captured graph."""
+    import os
+    import subprocess
+    import sys
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c", _SHRINKING_BATCH % (root, nx)], capture_output=True, text=True, timeout=300)
+    assert p.returncode == 0, p.stderr[-2000:]
