@@ -40,7 +40,7 @@ __device__ __forceinline__ double dot(const double (&u)[3], const double (&v)[3]
 
 }  // namespace
 
-// A block takes eb elements at a time, a thread the ns-th part of a line (fixed j, k) of one of them.
+// A block takes eb elements at a time (gridDim.y blocks share them), a thread the ns-th part of a line (fixed j, k) of one.
 __global__ void __launch_bounds__(kGeomThreads) k_geom(int64_t nelt, int nx, int eb, int ns, GllParams gp,
                                                        const double* __restrict__ corners, double* __restrict__ G)
 {
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kGeomThreads) k_geom(int64_t nelt, int nx, int
             for (int c = 0; c < 8; c++) sm[e][c][d] = v[c];
         }
         __syncthreads();
-        for (int q = threadIdx.x; q < ne * n2 * ns; q += kGeomThreads) {
+        for (int q = blockIdx.y * kGeomThreads + threadIdx.x; q < ne * n2 * ns; q += kGeomThreads * gridDim.y) {
             const int part = q / (ne * n2), ql = q - part * (ne * n2);
             const int e = ql / n2, l = ql - e * n2, k = l / nx, j = l - k * nx;
             const int len = (nx + ns - 1) / ns, i0 = part * len, i1 = min(nx, i0 + len);
@@ -125,14 +125,22 @@ extern "C" nek_status nek_geom(int64_t nelt, int nx, const double* corners, doub
     if (!corners || !G || !is_aligned(corners, 8) || !is_aligned(G, 16)) return NEK_ERR_INVALID_ARG;
     GllParams gp;
     gll_host(nx, gp.xi, gp.rho, nullptr);
-    // about two lines a thread and step, as many blocks as fit on the chip; fewer elements a block where that would leave
-    // SMs idle, and lines in parts where one element leaves threads idle (64 elements: nx = 4 14.2 us, 22.9 without;
-    // nx = 8 29.6, 39.5 without).  The values do not depend on either.
-    int eb = nx * nx >= 2 * kGeomThreads ? 1 : std::min(kGeomElems, 2 * kGeomThreads / (nx * nx));
+    // About two lines a thread and step, as many blocks as fit on the chip; fewer elements a block where that would leave
+    // SMs idle.  Lines in parts where one element leaves threads idle, and, up to half as many elements as SMs, until
+    // there is a thread for each on every SM; an element over several blocks where that makes more than one SM for it
+    // (one SM's FP64 pipe: nx = 16 needs 69 us for an element, 13.5 when a thread took one point; now 1 element 6.7 us, 64
+    // elements 36; nx = 10 6.4 and 15, 23.9 and 24 in one block an element).  More blocks or parts from 76 elements on
+    // are slower (100 elements of nx = 8 13.3 us with parts, 12.6 without).  The values do not depend on any of it.
+    const int n2 = nx * nx;
+    int eb = n2 >= 2 * kGeomThreads ? 1 : std::min(kGeomElems, 2 * kGeomThreads / n2);
     eb = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(eb, nelt / 152)));
-    const int ns = std::max(1, std::min(nx, kGeomThreads / (eb * nx * nx)));
+    int ns = kGeomThreads / (eb * n2);
+    if (nelt <= 76) ns = std::max(ns, 152 * kGeomThreads / (static_cast<int>(nelt) * n2));
+    ns = std::max(1, std::min(nx, ns));
     const int64_t nb = (nelt + eb - 1) / eb;
-    const int blocks = static_cast<int>(nb < 152 * 8 ? nb : 152 * 8);
-    k_geom<<<blocks, kGeomThreads, 0, static_cast<cudaStream_t>(stream)>>>(nelt, nx, eb, ns, gp, corners, G);
+    const int parts = static_cast<int>(
+        std::max<int64_t>(1, std::min<int64_t>((eb * n2 * ns + kGeomThreads - 1) / kGeomThreads, 2 * 152 / nb)));
+    const dim3 grid(static_cast<unsigned>(nb < 152 * 8 ? nb : 152 * 8), static_cast<unsigned>(parts));
+    k_geom<<<grid, kGeomThreads, 0, static_cast<cudaStream_t>(stream)>>>(nelt, nx, eb, ns, gp, corners, G);
     return check_launch();
 }

@@ -1067,3 +1067,19 @@ def test_batch_whose_fp64_launches_shrink_inside_captures(nx):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     p = subprocess.run([sys.executable, "-c", _SHRINKING_BATCH % (root, nx)], capture_output=True, text=True, timeout=300)
     assert p.returncode == 0, p.stderr[-2000:]
+
+
+@pytest.mark.parametrize("nx", [2, 6, 9, 10, 13, 15, 16])
+def test_geometry_bits_over_blocks_and_parts_of_lines(nx):
+    """Up to half as many elements as SMs a line goes to several threads and an element to several blocks: no bit of an
+    element's factors depends on it, and nothing is written beside them."""
+    mesh = inputs.box_mesh(14, 11, 1, nx, perturb=0.15, seed=nx)
+    c = _t(mesh.corners)
+    m = nx ** 3 * 6
+    G = torch.empty(mesh.nelt * m, dtype=torch.float64, device=DEV)
+    nekax.geom(mesh.nelt, nx, c, G)
+    for n in (1, 3, 8, 30, 64, 75, 76, 77, 100, 152, 153):
+        g = torch.full((n * m + 2,), float("nan"), dtype=torch.float64, device=DEV)
+        nekax.geom(n, nx, c[:n].contiguous(), g)
+        torch.cuda.synchronize()
+        assert torch.equal(g[:n * m], G[:n * m]) and torch.all(torch.isnan(g[n * m:]))
