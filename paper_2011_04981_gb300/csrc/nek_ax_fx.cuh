@@ -72,7 +72,8 @@ struct FxSmem {
     FxTab<NX> t1, t2;
     float rs[NX];           // phase 1: value of one unit of row i's sums
     unsigned mx[2][2 * (EPB + 1)];  // per element: bits of max |u|, of max |wr|, |ws|, |wt|; two buffers
-    int dexp[NX + 1];  // exponents above row i's absolute sum, and above the largest entry
+    int dexp[NX];      // exponents above row i's absolute sum
+    unsigned dmax;     // high word of the largest entry's magnitude
     double esum[fx_threads(NX, EPB)];
 };
 
@@ -138,23 +139,38 @@ __device__ __forceinline__ double fx_ldexp_any(long long z, int x)
 // The folded matrix of one phase.  M = D (phase 1) or D^T (phase 2).  Row i, entry l < ceil(n/2): the even part
 // multiplies u_l + u_{n-1-l} (the middle point alone where n is odd), the odd part u_l - u_{n-1-l}.  Values are
 // scaled by 2^(bits - E) with 2^E above the row's absolute sum (PER_ROW) or the matrix's largest entry, and split into
-// the nearest integer and the float remainder; the float forms are multiplied by unit[i] (PER_ROW) or 2^-kCrossShift.
+// the nearest integer and the float remainder; the float forms are multiplied by s: the value of one unit of the row's
+// sums (PER_ROW) or 2^-kCrossShift.  Entry q = i ceil(n/2) + l of the table, e its E.
 template <int NX, bool PER_ROW>
-__device__ __forceinline__ void fx_build(const double* Ds, int bits, const int* dexp, const float* unit,
-                                         FxTab<NX>& t, int tid, int nt)
+__device__ __forceinline__ void fx_entry(const double* Ds, int q, int e, float s, FxTab<NX>& t)
 {
-    constexpr int HE = FxTab<NX>::HE;
-    for (int q = tid; q < NX * HE; q += nt) {
-        const int i = q / HE, l = q - i * HE, m = NX - 1 - l;
-        const double a = PER_ROW ? Ds[i * NX + l] : Ds[l * NX + i];
-        const double b = PER_ROW ? Ds[i * NX + m] : Ds[m * NX + i];
-        const double sc = __hiloint2double((1023 + bits - (PER_ROW ? dexp[i] : dexp[NX])) << 20, 0);
-        const double ve = (l == m ? a : 0.5 * (a + b)) * sc, vo = (l == m ? 0.0 : 0.5 * (a - b)) * sc;
-        const int de = __double2int_rn(ve), dd = __double2int_rn(vo);
-        const float s = PER_ROW ? unit[i] : 1.f / (1 << kCrossShift);
-        t.f[q] = make_float4((float)(ve - (double)de) * s, (float)(vo - (double)dd) * s, (float)de * s, (float)dd * s);
-        t.d[i * FxTab<NX>::NI + 2 * l] = de;
-        t.d[i * FxTab<NX>::NI + 2 * l + 1] = dd;
+    constexpr int HE = FxTab<NX>::HE, kBits = PER_ROW ? kBits1 : kBits2;
+    const int i = q / HE, l = q - i * HE, m = NX - 1 - l;
+    const double a = PER_ROW ? Ds[i * NX + l] : Ds[l * NX + i];
+    const double b = PER_ROW ? Ds[i * NX + m] : Ds[m * NX + i];
+    const double sc = __hiloint2double((1023 + kBits - e) << 20, 0);
+    const double ve = (l == m ? a : 0.5 * (a + b)) * sc, vo = (l == m ? 0.0 : 0.5 * (a - b)) * sc;
+    const int de = __double2int_rn(ve), dd = __double2int_rn(vo);
+    t.f[q] = make_float4((float)(ve - (double)de) * s, (float)(vo - (double)dd) * s, (float)de * s, (float)dd * s);
+    t.d[i * FxTab<NX>::NI + 2 * l] = de;
+    t.d[i * FxTab<NX>::NI + 2 * l + 1] = dd;
+}
+
+// Both tables, an entry a thread.  An FP64 instruction takes a warp 64 clocks: the tables one after the other, and the
+// largest entry by a chain of nx^2 maxima in one thread, made every call 5 us longer at nx = 10 and 14 at nx = 16 (64
+// elements: nx = 10 15.0 -> 9.4 us, 8 10.8 -> 6.7, 16 32.6 -> 18.4).
+template <int NX>
+__device__ __forceinline__ void fx_build(const double* Ds, const int* dexp, int ED, FxTab<NX>& t1, FxTab<NX>& t2, int tid,
+                                         int nt)
+{
+    constexpr int N = NX * FxTab<NX>::HE;
+    for (int q = tid; q < 2 * N; q += nt) {
+        if (q < N) {
+            const int e = dexp[q / FxTab<NX>::HE];
+            fx_entry<NX, true>(Ds, q, e, pow2f(e - kBitsU - kBits1), t1);
+        } else {
+            fx_entry<NX, false>(Ds, q - N, ED, 1.f / (1 << kCrossShift), t2);
+        }
     }
 }
 
@@ -326,25 +342,28 @@ __global__ void __launch_bounds__(fx_threads(NX, EPB), (fx_min_blocks<NX, EPB>()
         double* Ds = reinterpret_cast<double*>(S.A);
         for (int q = tid; q < N2; q += NT) Ds[q] = D[q];
         if (tid < 2 * (EPB + 1)) S.mx[0][tid] = S.mx[1][tid] = 0u;
+        if (tid == 0) S.dmax = 0u;
         __syncthreads();
         bool asym = false;
-        for (int q = tid; q < N2; q += NT) asym = asym || Ds[q] != -Ds[N2 - 1 - q];
-        if (tid <= NX) {
+        unsigned hm = 0u;
+        for (int q = tid; q < N2; q += NT) {
+            asym = asym || Ds[q] != -Ds[N2 - 1 - q];
+            hm = max(hm, (unsigned)__double2hiint(Ds[q]) & 0x7FFFFFFFu);
+        }
+        hm = __reduce_max_sync(0xffffffffu, hm);
+        if ((tid & 31) == 0 && hm) atomicMax(&S.dmax, hm);
+        if (tid < NX) {
             double m = 0.0;
-            if (tid < NX)
-                for (int l = 0; l < NX; l++) m += fabs(Ds[tid * NX + l]);
-            else
-                for (int l = 0; l < N2; l++) m = fmax(m, fabs(Ds[l]));  // a NaN shows in its row's sum
-            S.dexp[tid] = max((__double2hiint(m) >> 20) - 1022, -100);
+            for (int l = 0; l < NX; l++) m += fabs(Ds[tid * NX + l]);
+            const int e = max((__double2hiint(m) >> 20) - 1022, -100);
+            S.dexp[tid] = e;
+            S.rs[tid] = pow2f(e - kBitsU - kBits1);
         }
         sym = !__syncthreads_or(asym);
-        if (tid < NX) S.rs[tid] = pow2f(S.dexp[tid] - kBitsU - kBits1);
-        ED = S.dexp[NX];
-        dbad = ED >= 128;  // beyond the float range, infinite
+        ED = max((int)(S.dmax >> 20) - 1022, -100);
+        dbad = ED >= 128;  // beyond the float range, infinite, NaN
         for (int l = 0; l < NX; l++) dbad = dbad || S.dexp[l] >= 132;
-        __syncthreads();
-        fx_build<NX, true>(Ds, kBits1, S.dexp, S.rs, S.t1, tid, NT);
-        fx_build<NX, false>(Ds, kBits2, S.dexp, S.rs, S.t2, tid, NT);
+        fx_build<NX>(Ds, S.dexp, ED, S.t1, S.t2, tid, NT);
         __syncthreads();
     }
 

@@ -1083,3 +1083,22 @@ def test_geometry_bits_over_blocks_and_parts_of_lines(nx):
         nekax.geom(n, nx, c[:n].contiguous(), g)
         torch.cuda.synchronize()
         assert torch.equal(g[:n * m], G[:n * m]) and torch.all(torch.isnan(g[n * m:]))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -1e60])
+@pytest.mark.parametrize("nx", [5, 10, 16])
+def test_ax_ff_matrix_beyond_the_float_range(nx, bad):
+    """An entry of D that is not finite, or beyond the float range, wherever it stands: no output is finite; a zero D gives
+    zero."""
+    rng = np.random.default_rng(nx)
+    xi, rho, D = ref.gll(nx)
+    mesh = inputs.box_mesh(3, 1, 1, nx, perturb=0.2, seed=nx)
+    G = _t(ref.geom(mesh.corners, nx, xi, rho))
+    u = _t(rng.uniform(-1, 1, size=(3, nx ** 3)))
+    for q in (0, nx + 1, nx * nx - 1):
+        E = D.copy()
+        E.reshape(-1)[q] = bad
+        w, _ = _ff_operator(nx, 3, _t(E), G, u)
+        assert not np.any(np.isfinite(w))
+    w, _ = _ff_operator(nx, 3, _t(np.zeros_like(D)), G, u)
+    assert np.all(w == 0.0)
