@@ -90,15 +90,18 @@ nek_status launch_diag_local(int64_t nelt, int nx, const double* D, const double
 {
     static std::atomic<uint64_t> configured{0};
     const int n2 = nx * nx, n3 = n2 * nx;
-    // elements a block stages: about two points a thread, within 100 KB
-    const int eb = std::max(1, std::min(2 * kDiagThreads / n3, 8));
+    // elements a block stages: about two points a thread, within 100 KB, and no more than it takes for a block on every SM
+    const int eb = static_cast<int>(
+        std::max<int64_t>(1, std::min<int64_t>(std::min(2 * kDiagThreads / n3, 8), (nelt + 151) / 152)));
     const size_t smem = sizeof(double) * (2 * n2 + (size_t)eb * 3 * n3);
     nek_status st = ensure_dyn_smem(k_diag_local, sizeof(double) * (2 * 256 + 3 * 4096), configured);  // nx = 16
     if (st != NEK_OK) return st;
     const int64_t nb = (nelt + eb - 1) / eb;
-    // several blocks on an element's points where there are fewer elements than SMs (64 elements of nx = 16: the call
-    // 47.3 us, 75.9 with one)
-    const int parts = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(eb * n3 / kDiagThreads, 2 * 152 / nb)));
+    // several blocks on a block's points, up to a point a thread, where there are SMs for them (64 elements of nx = 16: the
+    // call 41 us, 75.9 with one; 30 of nx = 10 11.2, 13.5 with as many as fill their threads; more than two an SM are
+    // slower), and three where a few SMs would have two elements and the others one (153 of nx = 10: 25.7, 29.8 with one)
+    const int most = (eb * n3 + kDiagThreads - 1) / kDiagThreads;
+    const int parts = static_cast<int>(nb <= 152 ? std::min<int64_t>(most, 2 * 152 / nb) : nb <= 200 ? std::min(most, 3) : 1);
     const dim3 grid(static_cast<unsigned>(std::min<int64_t>(nb, 152 * 8)), static_cast<unsigned>(parts));
     k_diag_local<<<grid, kDiagThreads, smem, s>>>(nelt, nx, eb, D, G, d);
     return check_launch();

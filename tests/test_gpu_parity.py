@@ -1102,3 +1102,27 @@ def test_ax_ff_matrix_beyond_the_float_range(nx, bad):
         assert not np.any(np.isfinite(w))
     w, _ = _ff_operator(nx, 3, _t(np.zeros_like(D)), G, u)
     assert np.all(w == 0.0)
+
+
+@pytest.mark.parametrize("nx", [2, 3, 5, 7, 10, 14, 16])
+def test_diagonal_bits_over_blocks(nx):
+    """The operator's diagonal on few elements (an element over several blocks), on a few more than SMs, and on many: no bit
+    of an element's values depends on how many there are."""
+    mesh = inputs.box_mesh(18, 17, 1, nx, perturb=0.15, seed=nx)
+    P = DeviceProblem(mesh, DEV, build_minv=False)
+    n3 = nx ** 3
+
+    def diag(n):
+        gs = nekax.GsPlan(n, nx, np.arange(n * n3, dtype=np.int64))
+        out = torch.full((n * n3 + 1,), 7.0, dtype=torch.float64, device=DEV)
+        nekax.jacobi_minv(gs, n, nx, P.D, P.G, torch.ones(n * n3, dtype=torch.uint8, device=DEV), out)
+        torch.cuda.synchronize()
+        assert out[-1] == 7.0
+        return out[:-1]
+
+    all_ = diag(mesh.nelt)
+    G, D = P.G[:2].cpu().numpy(), P.D_host
+    g = np.stack([np.array([ref.ax(D, G[e:e + 1], np.eye(n3)[q:q + 1])[0, q] for q in range(0, n3, 7)]) for e in range(2)])
+    assert _rel(1.0 / all_.cpu().numpy()[:2 * n3].reshape(2, n3)[:, ::7], g) <= 1e-13
+    for n in (1, 2, 30, 64, 100, 151, 152, 153, 200, 201):
+        assert torch.equal(diag(n), all_[:n * n3]), n
