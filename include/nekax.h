@@ -185,13 +185,17 @@ nek_status nek_ax_oz_selftest(int force_timeout, int64_t wait_us, int* timed_out
 
 /* ------------------------------------------------------------ tuning ---
  * The AX kernels group elements into CTAs; the group size (1, 2 or 4 elements
- * per CTA where threads and shared memory allow) changes only occupancy, never
- * the arithmetic, so results are bit-identical.  nek_tune_ax times each size on
+ * per CTA) changes only occupancy, never the arithmetic, so results are
+ * bit-identical.  It is what is asked for: a kernel that holds fewer, or on few
+ * elements always one, takes every size alike (NEK_AX_FP64 from nx = 9 on, and
+ * on no more elements than SMs).  nek_tune_ax times the built-in default and
+ * each size that runs another kernel on
  * the given data (synchronously; u, G/Gff, w as for nek_ax / nek_ax_ff with
  * impl = NEK_AX_FP64 / NEK_AX_FF, 16-byte aligned; the median of 7
  * individually timed launches) and keeps the fastest for all later launches of
- * that (impl, nx) in this process; *epb_out and *ms_out (nullable) receive it
- * and its time per launch.  For NEK_AX_FF the form with
+ * that (impl, nx) in this process, the default where none is faster; *epb_out
+ * and *ms_out (nullable) receive it (0: the default of NEK_AX_FP64 at nx = 2,
+ * which is none of the three) and its time per launch.  For NEK_AX_FF the form with
  * element energies that nek_cg_solve_ex uses is tuned too (kept on its own,
  * not reported).  nek_set_ax_epb sets the size
  * directly (0 restores the built-in default; a size that does not fit the

@@ -120,7 +120,8 @@ nek_status launch_ax_variant(int64_t nelt, const double* D, const double* G, con
     return check_launch();
 }
 
-// The elements-per-CTA counts that are accepted: 1, 2 and 4; at nx = 16 1 and 2.
+// The elements-per-CTA counts that are accepted: 1, 2 and 4; at nx = 16 1 and 2 (the set does not depend on the kernels
+// that run: see ax_fp64_form for which of them differ).
 constexpr bool ax_fits(int nx, int epb)
 {
     return (epb == 1 || epb == 2 || epb == 4) && nx * nx * epb <= 1024 &&
@@ -148,6 +149,14 @@ nek_status launch_ax_fp64_epb(int epb, int64_t nelt, int nx, const double* D, co
 }
 
 bool ax_fp64_epb_fits(int nx, int epb) { return nx >= kMinNx && nx <= kMaxNx && ax_fits(nx, epb); }
+
+int ax_fp64_default_epb(int nx) { return nx == 2 ? 0 : dx_default_epb(nx); }
+
+int ax_fp64_form(int64_t nelt, int nx, int epb)
+{
+    if (nx == 2) return epb > 0 ? epb : 32;
+    return nelt <= kSMs ? 0 : dx_conc(nx, epb > 0 ? epb : dx_default_epb(nx));
+}
 
 nek_status launch_ax_fp64(int64_t nelt, int nx, const double* D, const double* G, const double* u, double* w,
                           cudaStream_t s)

@@ -46,6 +46,8 @@ bool ax_ff_epb_fits(int nx, int epb)
     }
 }
 
+int ax_ff_default_epb(int nx) { return ff_epb(nx); }
+
 nek_status launch_ax_ff(int64_t nelt, int nx, const double* D, const float* Gff, const double* u, double* w,
                         cudaStream_t s, const int32_t* l2g, const int32_t* eprob, const uint8_t* pdone,
                         double* edot, const DirUpdate* dir)

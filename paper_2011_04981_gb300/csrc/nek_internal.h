@@ -56,7 +56,12 @@ void gll_host(int nx, double* xi, double* rho, double* D);
 constexpr int kAxFfEnergy = NEK_AX_FF_ENERGY;
 int tuned_epb(int impl, int nx);
 bool ax_fp64_epb_fits(int nx, int epb);
+// The kernel that epb (0: the default) stands for on nelt elements: counts of equal form run the same one.
+int ax_fp64_form(int64_t nelt, int nx, int epb);
+// The default count, 0 where it is none of 1, 2 and 4.
+int ax_fp64_default_epb(int nx);
 bool ax_ff_epb_fits(int nx, int epb);
+int ax_ff_default_epb(int nx);
 nek_status launch_ax_fp64_epb(int epb, int64_t nelt, int nx, const double* D, const double* G, const double* u,
                               double* w, cudaStream_t s);
 // l2g (optional): u is then a unique-node vector and element point p of the

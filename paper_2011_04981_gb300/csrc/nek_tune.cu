@@ -1,6 +1,6 @@
 // Elements-per-CTA selection for the AX kernels.
 //
-// Every AX kernel is compiled for several elements-per-CTA counts (1, 2, 4 where
+// The AX kernels are compiled for several elements-per-CTA counts (1, 2, 4 where
 // the thread count and shared memory allow).  The count changes only how
 // elements are grouped into CTAs, never the arithmetic on an element, so all
 // variants give bit-identical results; it trades occupancy against how much of
@@ -68,10 +68,17 @@ nek_status nek_tune_ax(int impl, int64_t nelt, int nx, const double* D, const vo
     float best_plain_ms = 0.f;
     const int nforms = impl == NEK_AX_FF ? 2 : 1;
     for (int form = 0; form < nforms && st == NEK_OK; form++) {
-        int best = 0;
+        int best = -1;
         float best_ms = 0.f;
-        const int cand[3] = {1, 2, 4};
-        for (int c = 0; c < 3 && st == NEK_OK; c++) {
+        // the built-in default first, so that it stays where no other is faster; then the other counts, without those that
+        // run a kernel already timed (of the FP64 operator: all of them on no more elements than SMs, and from nx = 9 on)
+        const int cand[4] = {impl == NEK_AX_FF ? ax_ff_default_epb(nx) : ax_fp64_default_epb(nx), 1, 2, 4};
+        for (int c = 0; c < 4 && st == NEK_OK; c++) {
+            bool seen = false;
+            for (int b = 0; b < c; b++)
+                seen = seen || cand[b] == cand[c] ||
+                       (impl == NEK_AX_FP64 && ax_fp64_form(nelt, nx, cand[b]) == ax_fp64_form(nelt, nx, cand[c]));
+            if (seen) continue;
             auto run = [&]() {
                 return impl == NEK_AX_FF
                            ? launch_ax_ff_epb(cand[c], nelt, nx, D, static_cast<const float*>(Gx), u, w, s, nullptr,
@@ -96,12 +103,12 @@ nek_status nek_tune_ax(int impl, int64_t nelt, int nx, const double* D, const vo
             for (int r = 0; r < kReps; r++) cudaEventElapsedTime(&t[r], ev[r], ev[r + 1]);
             std::sort(t, t + kReps);
             const float ms = t[kReps / 2];
-            if (best == 0 || ms < best_ms) {
+            if (best < 0 || ms < best_ms) {
                 best = cand[c];
                 best_ms = ms;
             }
         }
-        if (st == NEK_OK && best == 0) st = NEK_ERR_INVALID_ARG;
+        if (st == NEK_OK && best < 0) st = NEK_ERR_INVALID_ARG;
         if (st != NEK_OK) break;
         g_epb[form ? kAxFfEnergy : impl][nx].store(best, std::memory_order_relaxed);
         if (form == 0) {

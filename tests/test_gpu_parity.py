@@ -1126,3 +1126,31 @@ def test_diagonal_bits_over_blocks(nx):
     assert _rel(1.0 / all_.cpu().numpy()[:2 * n3].reshape(2, n3)[:, ::7], g) <= 1e-13
     for n in (1, 2, 30, 64, 100, 151, 152, 153, 200, 201):
         assert torch.equal(diag(n), all_[:n * n3]), n
+
+
+@pytest.mark.parametrize("nx,want", [(3, 2), (4, 4), (5, 4), (7, 2), (8, 1), (10, 1), (16, 1)])
+def test_tuning_where_every_count_runs_the_same_kernel(nx, want):
+    """On no more elements than SMs the FP64 operator has one kernel, whatever count is asked for: tuning there keeps the
+    built-in count for the larger calls.  From nx = 9 on that holds on any number of elements."""
+    for dims in ((4, 3, 3), (19, 4, 2)) if nx < 9 else ((4, 3, 3), (17, 5, 3)):
+        mesh = inputs.box_mesh(*dims, nx, perturb=0.1, seed=nx)
+        P = DeviceProblem(mesh, DEV, build_minv=False)
+        u = _t(inputs.random_local_field(mesh.nelt, nx, seed=3))
+        try:
+            epb, ms = nekax.tune_ax(nekax.AX_FP64, mesh.nelt, nx, P.D, P.G, u, torch.empty_like(u))
+            assert epb == want and ms > 0 and nekax.get_ax_epb(nekax.AX_FP64, nx) == want
+        finally:
+            nekax.set_ax_epb(nekax.AX_FP64, nx, 0)
+
+
+def test_tuning_times_the_default_of_order_2():
+    """The default of the FP64 operator at nx = 2 (32 elements a CTA) is none of the counts; on a large mesh it is far
+    ahead of them, and is kept."""
+    mesh = inputs.box_mesh(48, 48, 48, 2, perturb=0.1, seed=2)
+    P = DeviceProblem(mesh, DEV, build_minv=False)
+    u = _t(inputs.random_local_field(mesh.nelt, 2, seed=3))
+    try:
+        epb, ms = nekax.tune_ax(nekax.AX_FP64, mesh.nelt, 2, P.D, P.G, u, torch.empty_like(u))
+        assert epb == 0 and ms > 0 and nekax.get_ax_epb(nekax.AX_FP64, 2) == 0
+    finally:
+        nekax.set_ax_epb(nekax.AX_FP64, 2, 0)
