@@ -471,3 +471,29 @@ def test_prep_conversion_to_single_is_correctly_rounded(nelt):
     for ch in (0, 1):
         assert np.array_equal(xin[:, ch].cpu().numpy().view(np.uint32), want.view(np.uint32))
     assert torch.all(sc == 2.0 ** 35)
+
+
+def _sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("extra", [-1, 0, 1, 2, 1216, 1219])
+def test_apply_bf16_beyond_one_pass(extra):
+    """A pass of the inference kernel is four pairs of elements an SM.  From the second on a group reuses its tile, its
+    tensor-memory columns and its barrier's phase, with the input loaded ahead: every element's output is, to the bit, that
+    of calls small enough for one pass."""
+    n = 8 * _sms() + extra
+    rng = np.random.default_rng(100 + extra)
+    th = torch.from_numpy(_theta(9).astype(np.float32)).to(DEV)
+    xin = torch.from_numpy(rng.normal(size=(n, 2, 512)).astype(np.float32)).to(DEV)
+    sc = torch.from_numpy(rng.uniform(0.1, 2.0, size=n).astype(np.float32)).to(DEV)
+    c = torch.from_numpy(rng.uniform(0.1, 1.0, size=(n, 512))).to(DEV)
+    z = torch.full((n + 1, 512), -7.0, dtype=torch.float64, device=DEV)
+    nekax.net_apply_bf16(n, 8, th, xin, sc, c, z)
+    part = torch.full((n, 512), float("nan"), dtype=torch.float64, device=DEV)
+    step = 2 * _sms() - 1
+    for a in range(0, n, step):
+        b = min(n, a + step)
+        nekax.net_apply_bf16(b - a, 8, th, xin[a:b], sc[a:b], c[a:b], part[a:b])
+    torch.cuda.synchronize()
+    assert torch.all(z[n] == -7.0) and torch.all(torch.isfinite(z)) and torch.equal(z[:n], part)

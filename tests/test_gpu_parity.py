@@ -1154,3 +1154,55 @@ def test_tuning_times_the_default_of_order_2():
         assert epb == 0 and ms > 0 and nekax.get_ax_epb(nekax.AX_FP64, 2) == 0
     finally:
         nekax.set_ax_epb(nekax.AX_FP64, 2, 0)
+
+
+# ------------------------------------------------- reduced precision on the tensor cores, more elements than resident CTAs
+@pytest.mark.parametrize("prec", [nekax.PREC_BF16, nekax.PREC_F16])
+@pytest.mark.parametrize("nx", [2, 3, 5, 8, 9, 10, 11])
+def test_ax_lowp_tc5_beyond_the_resident_ctas(nx, prec):
+    """A CTA takes one element after another, with the next one's input loaded under the current one's second half (up to
+    nx = 10): every element's output is, to the bit, that of calls small enough for one element a CTA."""
+    base, n = 50, 2 * 8 * 152 + 3
+    mesh = inputs.box_mesh(base, 1, 1, nx, perturb=0.2, seed=nx)
+    P = DeviceProblem(mesh, DEV, build_minv=False)
+    G = P.G[torch.arange(n, device=DEV) % base].contiguous()
+    rng = np.random.default_rng(nx)
+    u = _t((rng.uniform(-1, 1, size=(n, nx ** 3)) * np.exp(rng.uniform(-5, 5, size=(n, 1)))).astype(np.float32))
+    Glp = torch.empty((n, nx ** 3, 6), dtype=torch.float16, device=DEV)
+    gsc = torch.empty(n, dtype=torch.float32, device=DEV)
+    nekax.geom_lowp(n, nx, prec, G, Glp, gsc)
+    w = torch.full((n + 1, nx ** 3), -7.0, dtype=torch.float32, device=DEV)
+    nekax.ax_lowp_tc5(n, nx, prec, P.D, Glp, gsc, u, w)
+    part = torch.full((n, nx ** 3), float("nan"), dtype=torch.float32, device=DEV)
+    for a in range(0, n, 151):
+        b = min(n, a + 151)
+        nekax.ax_lowp_tc5(b - a, nx, prec, P.D, Glp[a:b], gsc[a:b], u[a:b], part[a:b])
+    torch.cuda.synchronize()
+    assert torch.all(w[n] == -7.0) and torch.all(torch.isfinite(w)) and torch.equal(w[:n], part)
+
+
+@pytest.mark.parametrize("prec", [nekax.PREC_BF16, nekax.PREC_F16])
+@pytest.mark.parametrize("nx", [3, 8, 10, 11])
+def test_cg_mixed_beyond_the_resident_ctas(nx, prec):
+    """Defect correction on many copies of one element that share no node: the scalars are common to all, so every copy's x
+    is the same to the bit, whichever CTA and trip of the inner operator's persistent kernel (element energies, direction
+    update) it falls to."""
+    one = inputs.box_mesh(1, 1, 1, nx, perturb=0.2, seed=nx)
+    n, n3 = 8 * 152 + 5, nx ** 3
+    xi, rho, Dh = nekax.gll(nx)
+    D = _t(Dh)
+    G = torch.empty((n, n3, 6), dtype=torch.float64, device=DEV)
+    nekax.geom(n, nx, _t(np.tile(one.corners, (n, 1, 1))), G)
+    gs = nekax.GsPlan(n, nx, np.arange(n * n3, dtype=np.int64))
+    m = _t(np.tile(one.mask.reshape(1, n3), (n, 1)))
+    f = _t(np.tile(inputs.random_global_field(one, seed=4).reshape(1, n3), (n, 1)))
+    minv = torch.empty((n, n3), dtype=torch.float64, device=DEV)
+    nekax.jacobi_minv(gs, n, nx, D, G, m, minv)
+    Glp = torch.empty((n, n3, 6), dtype=torch.float16, device=DEV)
+    gsc = torch.empty(n, dtype=torch.float32, device=DEV)
+    nekax.geom_lowp(n, nx, prec, G, Glp, gsc)
+    x = torch.full((n, n3), float("nan"), dtype=torch.float64, device=DEV)
+    r = nekax.cg_solve_mixed(gs, n, nx, D, G, None, prec, Glp, gsc, m, minv, f, x, tol=1e-9, max_outer=30)
+    assert r["status"] == nekax.OK and r["inner"] >= r["outer"] >= 2
+    assert torch.all(torch.isfinite(x)) and float(x.abs().max()) > 0.0
+    assert torch.equal(x, x[:1].expand(n, n3))
