@@ -5,10 +5,11 @@ One step is one ``nek_cg_solve`` call of 100 Jacobi-PCG iterations (tol = 0, a
 fixed iteration count), i.e. 100 passes of the whole solve path: AX, dssum,
 mask, the weighted dot products and the vector updates.  ``value`` is local
 grid points x iterations per second (GDOF/s) over all ranks, with the
-FP64-accurate float-float operator.  The AX kernel is timed inside the same
-region with CUDA events on the solve's stream; it gives the roofline entry.
-``e2e`` times the same steps through ``nek_cg_solve_host`` (f and x in pinned
-host memory, both copies inside the call).
+FP64-accurate operator of the integer and FP32 pipes (``nek_ax_ff``, "float-float"
+below).  The AX kernel is timed inside the same region with CUDA events on the
+solve's stream; it gives the roofline entry.  ``e2e`` times the same steps
+through ``nek_cg_solve_host`` (f and x in pinned host memory, both copies inside
+the call).
 
 The default run also carries the rest of the metric (rank 0, after the timed
 region): the same solve with the native FP64 operator, the standalone AX sweep
@@ -677,8 +678,7 @@ def tensor_core_block(torch, P, f, x, ws, iters, steps=3):
     hbm, kind = peaks()
     t_ax = out["ax"]["ms_per_launch"] / 1e3
     out["ax"].update({"kernel": "k_ax_oz<%d, 2>" % P.nx, "hbm_frac_104B": 104 * P.npts / t_ax / 1e9 / hbm})
-    out["note"] = ("FP64-accurate; HBM %s %.0f GB/s.  Standalone (64 B/point) this operator is faster than the "
-                   "float-float one (ax_sweep), inside the solve its fused update's FP64 operations (x and p "
+    out["note"] = ("FP64-accurate; HBM %s %.0f GB/s.  Inside the solve its fused update's FP64 operations (x and p "
                    "updates, energies, the join to FP64: 5 per point on the 2-per-clock FP64 pipe) are not "
                    "hidden by its two CTAs per SM" % (kind, hbm))
     return out
@@ -814,18 +814,19 @@ def run_native(args):
     # the float-float operator of the solve also applies the x / direction update
     fused_dir = args.ax in ("ff", "oz")
     ax_bpp = 104 if fused_dir else 64
+    ff_arith = "block fixed point on the integer and FP32 pipes" if nx >= 5 else "float-float on the FP32 pipes"
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": 1000 * t_dev / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
-        "dtype": {"fp64": "f64", "ff": "f64 (AX in f32-pair float-float, FP64-accurate)",
+        "dtype": {"fp64": "f64", "ff": "f64 (AX FP64-accurate, %s)" % ff_arith,
                   "oz": "f64 (AX contractions as BF16 digit slices on tcgen05 with exact FP32 level sums, "
                         "FP64-accurate)"}[args.ax],
         "data": "synthetic",
         "config": {"workload": "Jacobi-PCG, %d PCG iterations per step (AX+dssum+mask+dots+updates), "
                                "%dx%dx%d deformed box (perturbation 0.1 h), nx=%d, FP64-accurate, AX %s"
                                % (iters, e, e, e, nx, {"fp64": "native FP64 (nek_ax)",
-                                                       "ff": "float-float on the FP32 pipes (nek_ax_ff)",
+                                                       "ff": ff_arith + " (nek_ax_ff)",
                                                        "oz": "contractions on the tensor cores (nek_ax_oz)"}[args.ax]),
                    "elements": mesh.nelt, "nx": nx, "points": pts, "iters_per_step": iters,
                    "parallelism": "replicas" if world > 1 else "single",
@@ -850,10 +851,9 @@ def run_native(args):
                                  "k_ax_fx<%d>" if nx >= 5 else "k_ax_ff<%d>") % nx,
                       "note": ("FP64-accurate AX (%s) with the fused x / direction update, 104 algorithmic "
                                "B/point (p in and out 16, r 8, minv 8, x in and out 16, G 48, w 8)"
-                               % ("tensor-core digit slices" if args.ax == "oz" else "float-float") if fused_dir else
-                               "FP64-accurate float-float AX, 64 algorithmic B/point (u 8 + G 48 + w 8)") +
-                              "; peak = %s HBM copy (MEASURED_PEAKS hbm_gbs); its instruction limit is the FP32 "
-                              "pipe (see profiles)" % hbm_kind}),
+                               % ("tensor-core digit slices" if args.ax == "oz" else ff_arith) if fused_dir else
+                               "FP64-accurate AX, 64 algorithmic B/point (u 8 + G 48 + w 8)") +
+                              "; peak = %s HBM copy (MEASURED_PEAKS hbm_gbs); see profiles" % hbm_kind}),
         "clocks": clk,
     }
     ex = args.extra_set if rank == 0 else set()

@@ -54,7 +54,7 @@ typedef enum {
 /* Which AX operator a call uses. */
 typedef enum {
     NEK_AX_FP64 = 0,      /* nek_ax: FP64 */
-    NEK_AX_FF = 1,        /* nek_ax_ff: FP64-accurate float-float on the FP32 pipes; needs Gff */
+    NEK_AX_FF = 1,        /* nek_ax_ff: to FP64 accuracy on the integer and FP32 pipes (float-float); needs Gff */
     NEK_AX_FF_ENERGY = 2, /* nek_ax_ff's element-energy form (nek_ax_ff_energy and the solves):
                              for nek_set_ax_epb / nek_get_ax_epb only */
     NEK_AX_OZ = 3         /* nek_ax_oz: FP64-accurate with the contractions on the tensor cores; needs
@@ -100,7 +100,9 @@ nek_status nek_geom(int64_t nelt, int nx, const double* corners, double* G, void
  *   D: device, nx*nx; G: device, nelt*nx^3*6; u: device, in; w: device, out.
  *   u and w must not overlap.  Async on stream.
  * To FP64 rounding: from nx = 3 on the contractions are summed in 58-bit block fixed point per line (integers; lines that
- * are not finite or beyond 2^+-400 in FP64), the product with G in FP64; nx = 2 in FP64 throughout.
+ * are not finite or beyond 2^+-400 in FP64), the product with G in FP64; nx = 2 in FP64 throughout.  A line's sum is good to
+ * (2 nx + 4) 2^-57 of its largest value times D's row sum of magnitudes (a value more than 2^5 below the largest holds
+ * fewer than 53 bits), which a chain of FP64 operations betters only where D is zero or small at the line's largest value.
  */
 nek_status nek_ax(int64_t nelt, int nx, const double* D, const double* G, const double* u, double* w,
                   void* stream);
@@ -115,13 +117,14 @@ nek_status nek_ax(int64_t nelt, int nx, const double* D, const double* G, const 
 nek_status nek_geom_ff(int64_t nelt, int nx, const double* G, float* Gff, void* stream);
 
 /*
- * w = AX(u) to FP64 accuracy computed on the FP32 pipes (the operator of
- * Section II-B, Listing 1, in float-float arithmetic).  Same arguments and
+ * w = AX(u) to FP64 accuracy computed on the FP32 and, from nx = 5 on, the
+ * integer pipes (the operator of Section II-B, Listing 1).  Same arguments and
  * layouts as nek_ax except Gff (from nek_geom_ff); u, w 8-byte aligned, no
  * overlap.  Values are carried as pairs of floats (~48 significant bits) or, from
  * nx = 5 on, as integer digits of the element's largest value with float
- * remainders whose products are summed exactly; the result matches the
- * FP64 operator to ~1e-13 relative in the max norm.  Element blocks whose
+ * remainders whose products are summed exactly (a value below 2^-28 of the
+ * element's largest holds one float, 24 bits); the result matches the
+ * FP64 operator to ~1e-13 relative in the max norm of each element.  Element blocks whose
  * largest |u| is below ~1e-30 (or contain non-finite values) are not covered by
  * that accuracy statement.  Async on stream.
  */
@@ -558,7 +561,9 @@ size_t nek_cg_workspace_bytes(int64_t nelt, int nx, int need_minv);
 
 typedef struct {
     int check_every;     /* residual read-back period in iterations (>=1; default 1); the result does not depend on it */
-    int time_ax;         /* nonzero: record CUDA events around every AX launch */
+    int time_ax;         /* nonzero: record CUDA events around every AX launch.  An FP64 solve of few elements, one
+                            launch without it, then runs as the loop of launches: the same operations on every
+                            point, the sums in another order */
     double ax_ms_total;  /* out: summed AX kernel time when time_ax */
     int ax_launches;     /* out: number of AX launches */
     int kernel_launches; /* out: kernels this call enqueued */

@@ -11,12 +11,17 @@
 // multiply-adds (IMAD.WIDE) per clock take the contractions instead, in block fixed point per line, with FP64 for G:
 //   - a line's values become 58-bit integers at the scale of its largest, a matrix row 58-bit integers at the scale of
 //     its absolute sum, each as two 29-bit digits;
-//   - the high digits' products and the two cross products are summed exactly in 64 bits; the product of the low digits,
-//     below 2^-58 of the line's bound, is dropped.  The sum is rounded to a double by shifts (dx_ldexp);
+//   - the high digits' products and the two cross products are summed exactly in 64 bits; the products of the low digits,
+//     each below 2^-58 of the line's bound, are dropped.  The sum is rounded to a double by shifts (dx_ldexp);
 //   - D of a symmetric rule satisfies D[n-1-i][n-1-l] = -D[i][l]: with the sums and differences of mirrored points every
 //     product serves two outputs.  The kernel checks that of the D it is given and otherwise computes every row.
-// A result's error is below 2^-54 of its size plus about 2^-57 of the line's bound, where a chain of nx FP64 multiply-adds
-// has up to nx 2^-53 of it.  Measured against 128-bit arithmetic (2-norm, deformed boxes, random u; FP64 form in
+// A result's error is at most 2^-53 of its size (the final rounding) plus (2 nx + 4) 2^-57 of the line's largest value times
+// the row's absolute sum: the values' digits are truncated (2 of these), the matrix's rounded (nx), the low digits'
+// products dropped (nx + 1), the cross sums rounded (1).  An exact integer model gives up to 1.4 2^-57 at nx = 8 and 1.7 2^-57
+// at 16 (150 lines each, random, nearly equal and smooth).  A chain of nx FP64 multiply-adds has up to nx 2^-53 of the sum of
+// the terms' magnitudes; that is less only where D has a zero or small entry at a line's largest value (the zero diagonal of
+// a rule: a derivative there is good to 2^-57 of the line, not of its own size), and the sum of the three directions then
+// has larger terms from the same line.  Measured against 128-bit arithmetic (2-norm, deformed boxes, random u; FP64 form in
 // brackets): nx = 4 1.0e-16 (1.2e-16), 8 0.9e-16 (2.0e-16), 16 1.1e-16 (2.7e-16); smooth u, whose derivatives cancel: nx = 8
 // 2.4e-16 (1.8e-15).  Lines that are not finite, or outside 2^+-400, are summed in FP64 as they stand, and every line is if a
 // row of D is outside.
@@ -25,10 +30,10 @@
 // all their outputs; G and the result are point-wise over the same threads.  CTAs are persistent, the next element's
 // input is copied to shared memory (cp.async) under the current one's second half, G fetched into L2 during phase 1.
 //
-// What bounds it (nx = 8, 8000 elements, ncu): the FP64 pipe is 59 % busy with the G product (9 operations a point; 4.5
-// clocks, 64 us of the 131), the issue slots 54 %, ALU 52 %; the rest is the latency of the phases between the barriers of
-// 8 CTAs an SM.  408 -> 131 us; nx = 5 97 -> 49, 16 5.71 -> 1.64 ms (8000 elements), nx = 4 at 196608 elements 709 -> 503.
-// 64 elements at nx = 8 30 -> 8 us (launch list).
+// What bounds it (nx = 8, 8000 elements, ncu): the FP64 pipe is 63 % busy with the G product (9 operations a point; 4.5
+// clocks, 64 us of the 122), the issue slots 51 %, ALU 52 %; the rest is the latency of the phases between the barriers of
+// 8 CTAs an SM.  412 -> 122 us; nx = 5 97 -> 49, 16 5.71 -> 1.64 ms (8000 elements), nx = 4 at 196608 elements 709 -> 503.
+// 64 elements at nx = 8 30 -> 6.8 us.
 #pragma once
 
 #include "nek_internal.h"
@@ -40,8 +45,10 @@ namespace {
 
 // Lines per thread where elements fill the chip, and the resident warps per SM that the register budget is set for.  Two
 // lines share the loads of the matrix tables (nx = 8 128 against 141 us, 13 168 against 195, 15 221 against 229); at nx = 16
-// the block of 12 warps that would leave is slower (232 against 226).  Warps: nx = 8 128 us with 24, 142 with 20, 131 with
-// 30; nx = 10 156 with 28, 160 with 24, 170 with 30 (4.1 million points each).
+// the block of 12 warps that would leave is slower (232 against 226).  Warps (us, 8 million points): up to nx = 7 32 (nx = 5
+// 277, 288 with 28; 7 285, 291); 8 24 or 28 (233; 254 with 20, 237 with 32); 12, 13 and 15 24 and more alike (336, 327, 424;
+// 355, 336, 461 with 20); 9 and 10 277 and 292 with 28, 268 and 287 with 24 (nx = 10 at 4.1 million points 156 with 28, 160
+// with 24); 14 and 16 the same from 20 on (shared memory).
 constexpr int dx_lpt(int nx) { return nx <= 15 ? 2 : 1; }
 constexpr int dx_warps(int nx) { return nx <= 7 ? 32 : nx == 8 || nx == 12 || nx == 13 || nx >= 15 ? 24 : 28; }
 constexpr int dx_tpe(int nx, int lpt) { return (3 * nx * nx + lpt - 1) / lpt; }
@@ -87,8 +94,8 @@ __device__ __forceinline__ double dx_ldexp(long long z, int x)
     return __hiloint2double((int)((int)(g >> 32) >= 0 ? 0u : hi | ((unsigned)sg & 0x80000000u)), (int)(unsigned)m);
 }
 
-// Copies the matrix Dg to D, finds out whether it is symmetric as above, and fills t[0] (M = D) and t[1] (M = D^T), in integers (an FP64 chain here would be a third of the time of a call on few
-// elements).  Returns whether a row's absolute sum is outside kDxRange; the tables are then not to be used.
+// Copies the matrix Dg to D, finds out whether it is symmetric as above, and fills t[0] (M = D) and t[1] (M = D^T), in
+// integers (an FP64 chain here would be a third of the time of a call on few elements).  Returns whether a row's absolute sum is outside kDxRange; the tables are then not to be used.
 template <int NX>
 __device__ __forceinline__ bool dx_build(const double* __restrict__ Dg, double* D, DxTab<NX>* t, int tid, int nt, bool& sym)
 {
@@ -168,7 +175,7 @@ __device__ __forceinline__ void dx_lines(const double* const (&src)[LPT], double
         }
         const unsigned E = mx & 0x7FF00000u;
         ex[q] = (int)(E >> 20) - (1023 + 2 * kDxDigit);
-        // |v| as an integer of 56 bits at the scale of the line's largest, in two digits with v's sign
+        // |v| as an integer of 58 bits at the scale of the line's largest (truncated), in two digits with v's sign
         auto conv = [&](double x, int& h, int& l) {
             const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
             const unsigned s = (E - (hi & 0x7FF00000u)) >> 20;
@@ -395,7 +402,7 @@ __global__ void __launch_bounds__(dx_threads(NX, EPB, LPT), (dx_min_blocks<NX, E
 // us with 1, 2 and 4) and one is held.
 constexpr int dx_conc(int nx, int epb) { return nx >= 9 ? 1 : epb; }
 
-// The fastest of 1, 2 and 4 (8000 elements, us: nx = 5 49 with 4, 62 with 1; 7 111 with 2, 123 with 1; 8 131 with 1, 146
+// The fastest of 1, 2 and 4 (8000 elements, us: nx = 5 49 with 4, 62 with 1; 7 111 with 2, 123 with 1; 8 122 with 1, 146
 // with 2).
 constexpr int dx_default_epb(int nx) { return nx == 3 || nx == 7 ? 2 : nx <= 5 ? 4 : 1; }
 

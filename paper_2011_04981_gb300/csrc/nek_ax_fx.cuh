@@ -44,8 +44,11 @@ namespace {
 // Lines per thread (of the 3 nx^2 lines of a phase), resident warps per SM that the register budget is set for, and points
 // whose geometric factors are in flight together.  Two lines a thread halve the loads of the matrix tables; at nx = 11,
 // 12 and 14 one line with more warps measured faster (nx = 12: 0.71 against 0.74 ms plain, 0.92 against 0.98 with the
-// direction update, a 30-million-point launch).  Warps: nx = 10 0.59 ms with 20, 0.64 with 15, 0.79 with 25 (which spills);
-// nx = 8 0.28 with 24, 0.30 with 20.
+// direction update, a 30-million-point launch).  Warps (us, plain, 8 million points): nx = 6 145 with 28, 148 with 20; 8 139
+// with 24, 149 with 20, 151 with 28; 11 193 with 36, 191 with 28, 242 with 20; 12 183 with 28, 231 with 24; at the others 20,
+// where 16 is slower or the same (nx = 5 172 and 193, 7 169 and 182) and 28 is slower (9 162 and 191, 10 156 and 201, which
+// spills) or makes no difference (from 13 on: shared memory).  Points of G together, 2 or 3 (with energies): nx = 8 153 and
+// 149, 10 no difference, 6, 9 and 12 to 14 two to 6 % slower with three (9: 170 and 176).
 constexpr int fx_lpt(int nx) { return nx == 11 || nx == 12 || nx == 14 ? 1 : 2; }
 constexpr int fx_warps(int nx) { return nx == 6 || nx == 12 ? 28 : nx == 8 ? 24 : nx == 11 ? 36 : 20; }
 constexpr int fx_ahead(int nx) { return nx == 8 || nx == 10 ? 3 : 2; }

@@ -1,4 +1,4 @@
-// Shared by the line-pass AX kernels (nek_ax_fx.cuh, nek_ax.cu): the shared-memory layout of an element whose threads walk
+// Shared by the line-pass AX kernels (nek_ax_fx.cuh, nek_ax_dx.cuh): the shared-memory layout of an element whose threads walk
 // its lines, asynchronous copies, and the integer arithmetic of their block fixed point.
 #pragma once
 

@@ -10,10 +10,10 @@
 // tap (dj, dk) is one descriptor with the strides LBO = 2592 B, SBO = 144 B, shifted by
 // 16 (1 + dj) + 288 (1 + dk).  The three taps along i go to N: the MMA of input point i multiplies by a 16 x 48
 // operand (di = +1, 0, -1) into the TMEM columns of the output points i - 1, i and i + 1 (16 channels each, 128 columns
-// a tile): 78 MMAs a layer and two elements, where one MMA per tap takes 270 of N = 16.  An MMA of so few columns takes the time to read its 4 KB of A from shared memory, so the reads are
-// what counts.  Every output still sums its 27 taps in the order (dk, dj, di), one MMA each: the sums are
-// bit-identical to those of one MMA per tap.  The first (dj, dk) overwrites: the point i + 1 that an MMA reaches
-// first is a 16-column MMA of its own there.
+// a tile): 78 MMAs a layer and two elements, where one MMA per tap takes 270 of N = 16.  An MMA of so few columns takes
+// the time to read its 4 KB of A from shared memory, so the reads are what counts.  Every output still sums its 27 taps
+// in the order (dk, dj, di), one MMA each: the sums are bit-identical to those of one MMA per tap.  The first (dj, dk)
+// overwrites: the point i + 1 that an MMA reaches first is a 16-column MMA of its own there.
 //
 // A CTA has four groups of eight warps, each with its own tile (41 KB of activations, 128 TMEM columns) and
 // mbarrier; the weights (41 KB) are shared.  A group is a chain of MMAs, wait and epilogue per layer; the groups'
