@@ -31,7 +31,7 @@
 // input is copied to shared memory (cp.async) under the current one's second half, G fetched into L2 during phase 1.
 //
 // What bounds it (nx = 8, 8000 elements, ncu): the FP64 pipe is 63 % busy with the G product (9 operations a point; 4.5
-// clocks, 64 us of the 122), the issue slots 51 %, ALU 52 %; the rest is the latency of the phases between the barriers of
+// clocks, 64 us of the 122), the issue slots 50 %, ALU 52 %; the rest is the latency of the phases between the barriers of
 // 8 CTAs an SM.  412 -> 122 us; nx = 5 97 -> 49, 16 5.71 -> 1.64 ms (8000 elements), nx = 4 at 196608 elements 709 -> 503.
 // 64 elements at nx = 8 30 -> 6.8 us.
 #pragma once
@@ -95,7 +95,8 @@ __device__ __forceinline__ double dx_ldexp(long long z, int x)
 }
 
 // Copies the matrix Dg to D, finds out whether it is symmetric as above, and fills t[0] (M = D) and t[1] (M = D^T), in
-// integers (an FP64 chain here would be a third of the time of a call on few elements).  Returns whether a row's absolute sum is outside kDxRange; the tables are then not to be used.
+// integers (an FP64 chain here would be a third of the time of a call on few elements).  Returns whether a row's absolute
+// sum is outside kDxRange; the tables are then not to be used.
 template <int NX>
 __device__ __forceinline__ bool dx_build(const double* __restrict__ Dg, double* D, DxTab<NX>* t, int tid, int nt, bool& sym)
 {
@@ -144,8 +145,8 @@ __device__ __forceinline__ bool dx_build(const double* __restrict__ Dg, double* 
     return false;
 }
 
-// One line pass over LPT lines of NX points: src[q] and dst[q] hold NX values at stride st[q]; sg[q] is the sign bit to apply to
-// the input.
+// One line pass over LPT lines of NX points: src[q] and dst[q] hold NX values at stride st[q]; sg[q] is the sign bit to
+// apply to the input.
 template <int NX, bool TRANS, int LPT>
 __device__ __forceinline__ void dx_lines(const double* const (&src)[LPT], double* const (&dst)[LPT], const int (&st)[LPT],
                                          const unsigned (&sg)[LPT], const DxTab<NX>& tab, const double* D, bool sym, bool bad)
@@ -180,7 +181,8 @@ __device__ __forceinline__ void dx_lines(const double* const (&src)[LPT], double
             const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
             const unsigned s = (E - (hi & 0x7FF00000u)) >> 20;
             const unsigned mh = (hi & 0x000FFFFFu) | 0x00100000u;
-            const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 2 * kDxDigit - 53) << 32) | (lo << (2 * kDxDigit - 53));
+            constexpr int kUp = 2 * kDxDigit - 53;
+            const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, kUp) << 32) | (lo << kUp);
             unsigned long long a, b;
             asm("shr.u64 %0, %1, %2;" : "=l"(a) : "l"(m), "r"(s + kDxDigit));
             asm("shr.u64 %0, %1, %2;" : "=l"(b) : "l"(m), "r"(s));

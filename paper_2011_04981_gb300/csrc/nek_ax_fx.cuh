@@ -25,8 +25,8 @@
 //
 // What bounds it (nx = 10, 32768 elements, ncu): no unit is saturated; issue 52 %, shared-memory data path 61 %, FMA
 // pipes 36 %; the 4.8 warps a scheduler wait on fixed latencies, global loads, shared loads and barriers in about equal
-// parts.  0.62 ms = 53 GDOF/s = 0.50 of the measured HBM copy rate at 64 B/point (float-float item kernel before: 0.96
-// ms); with the solve's direction update 0.82 ms = 0.61 of it at 104 B/point (1.04 ms before).
+// parts.  0.61 ms = 53 GDOF/s = 0.50 of the measured HBM copy rate at 64 B/point (float-float item kernel before: 0.96
+// ms); with the solve's direction update 0.80 ms = 0.62 of it at 104 B/point (1.04 ms before).
 #pragma once
 
 #include <type_traits>

@@ -124,7 +124,8 @@ __device__ __forceinline__ void prob_sum2(const double* __restrict__ parts, int 
 }
 
 __global__ void __launch_bounds__(PT) kb_init_finish(const int* __restrict__ pch, const double* __restrict__ parts,
-                                                     int nchunks, double tol, BScal* __restrict__ sc, int* __restrict__ active)
+                                                     int nchunks, double tol, BScal* __restrict__ sc,
+                                                     int* __restrict__ active)
 {
     const int pid = blockIdx.x;
     double rz, rr;
@@ -172,8 +173,8 @@ __global__ void __launch_bounds__(BT) kb_pw(const int64_t* __restrict__ ch_begin
 // pw from the chunk partials of kb_pw or, with edot, from the element energies
 // of the float-float operator (problem p's elements are [pel[p], pel[p+1]))
 __global__ void __launch_bounds__(PT) kb_alpha(const int* __restrict__ pch, const double* __restrict__ parts,
-                                               BScal* __restrict__ sc, int* __restrict__ active, const int64_t* __restrict__ pel,
-                         const double* __restrict__ edot)
+                                               BScal* __restrict__ sc, int* __restrict__ active,
+                                               const int64_t* __restrict__ pel, const double* __restrict__ edot)
 {
     const int pid = blockIdx.x;
     if (bhalted(sc[pid])) {

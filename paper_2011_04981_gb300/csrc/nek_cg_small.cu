@@ -10,7 +10,7 @@
 // Every CTA adds the same partials in the same order, so all hold the same scalars and take the same exit; the host reads
 // them once.  The operations on a point are those of the kernels in nek_pcg.cuh.
 //
-// A call of 64 elements of nx = 8 takes 16.6 us an iteration (53 us as 7 launches and a read-back, 43 with a read-back every
+// A call of 64 elements of nx = 8 takes 15.3 us an iteration (53 us as 7 launches and a read-back, 43 with a read-back every
 // tenth); 456 elements of nx = 8 26 (60), 150 of nx = 5 16 (60), of nx = 16 57 (84), general loop timed with read-backs every
 // tenth iteration and events; faster on every size that fits, so the rule is that it fits.  What bounds it is latency, in
 // clocks of 32000 an iteration (64 elements, nx = 8): operator 10000, waits at the barriers 8500, sums over copies and

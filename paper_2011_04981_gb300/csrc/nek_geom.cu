@@ -10,8 +10,8 @@
 // x = sum m_abc r^a s^b t^c (a, b, c = 0, 1).  Along a line of points in r, x_r is constant, x_s and x_t are linear, hence
 // so are x_t x x_r and x_r x x_s: a thread forms their coefficients once for its line, and a point costs 21 operations up
 // to the three products and |J| instead of 99 (72 of them for the columns from the corners), 18 for the dot products and
-// a division.  24^3 elements at nx = 10: 1.5 ms, 4.1 before.  (x_s x x_t and |J| as quadratics in r saved three more
-// operations, and cost accuracy where |J| is small.)
+// a division.  24^3 elements at nx = 10: 1.6 ms, 4.1 before; the FP64 pipe is 92 % busy.  (x_s x x_t and |J| as
+// quadratics in r saved three more operations, and cost accuracy where |J| is small.)
 #include <algorithm>
 
 #include "nek_internal.h"

@@ -23,11 +23,12 @@
 // rounds to BF16 and writes the rows back in place (the next layer's input; every MMA of the layer has
 // completed by then).  The last layer writes z = y * scale * c in FP64.
 //
-// What bounds it (13 824 elements, 362 us against 975 before; 322 TFLOP/s of useful work): the MMAs alone, with
-// the GELUs left out, take 263 us, about 50 cycles each for the 42 shared-memory wavefronts of their operands; the GELUs alone
-// (25 instructions, ten of them on the half-rate ALU pipe) about 200 us of issue.  Three groups of four warps took
-// 500 us, three of eight 440, four of eight 418, and 362 once one elected thread issues all MMAs with operands in
-// uniform registers (20 instructions an MMA before, which the issuing warp did not get through between the GELUs).
+// What bounds it (13 824 elements, 362 us against 975 before; 320 TFLOP/s of useful work; tensor pipe 33 %, issue
+// 53 %): the MMAs alone, with the GELUs left out, take 263 us, about 50 cycles each for the 42 shared-memory wavefronts of
+// their operands; the GELUs alone (25 instructions, ten of them on the half-rate ALU pipe) about 200 us of issue.  Three
+// groups of four warps took 500 us, three of eight 440, four of eight 418, and 362 once one elected thread issues all MMAs
+// with operands in uniform registers (20 instructions an MMA before, which the issuing warp did not get through between
+// the GELUs).
 //
 // Numerics are those of nek_net_apply_bf16's contract: BF16 weights, the input
 // and both hidden activations rounded to BF16 (nearest even) before each

@@ -8,7 +8,7 @@
 //
 // After anything that is not a kernel, or under a tool that serialises, the launch is an ordinary one and pdl_wait()
 // returns at once.  FP16 defect correction on 16^3 elements of nx = 10 (1655 iterations of
-// 5 launches): 160 -> 144 ms; 20 iterations on 24^3 elements 10.5 -> 10.25 ms.
+// 5 launches): 160 -> 148 ms; 20 iterations on 24^3 elements 10.5 -> 10.2 ms.
 #pragma once
 
 #include <cuda_runtime.h>
